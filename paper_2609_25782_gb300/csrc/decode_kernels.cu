@@ -13,6 +13,8 @@
 //                          (one warp per query head from registers, up to 16
 //                          splits; else four warps per head), launched as a
 //                          programmatic dependent of the split kernel.
+//   decode_combine_sub_kernel
+//                          the same where several CTAs shared each split.
 //
 // Hot pool: hot[NB][L][2][Hkv][bt][128] bf16. A (block, layer, K|V, head)
 // run is bt rows of 256 B, row = ((blk*L + l)*2 + kv)*Hkv + g)*bt + slot. The
@@ -20,6 +22,8 @@
 // K|V) and loads one box per 16-token tile: its 16 K rows and 16 V rows.
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
+
+#include <type_traits>
 
 #include "kvt_internal.h"
 
@@ -45,16 +49,19 @@ constexpr int kTileBytes = 8192;           // K 4 KiB + V 4 KiB
 constexpr int kHalfBytes = 2048;           // 16 rows x 128 B (64 dims)
 // The plan of one split: its tiles are dealt round robin to kAccs running
 // softmax states (accumulator v takes tiles v, v + kAccs, ...), which merge
-// in the order v = 0 .. kAccs-1 at the end. That plan fixes the result; how
-// the accumulators map to warps is a launch choice:
-//   <4 warps, KVT_STAGES slots>  3 CTAs per SM; a warp owns accumulators w
-//                                and w + 4 and alternates between them, so
-//                                consecutive tiles of a warp are independent
-//   <4 warps, 3 slots>           2 CTAs per SM
-//   <8 warps, 3 slots>           1 CTA per SM (small grids): one accumulator
-//                                per warp, twice the warps per SM
-// Each SM keeps about 24 tiles in flight whatever the variant, and every
-// variant gives bit-identical results.
+// as a tree of neighbours (0 1, 2 3, ...; then pairs of pairs) at the end.
+// That plan fixes the result; how the accumulators map to warps and CTAs is a
+// launch choice, and every choice gives bit-identical results:
+//   <4 warps, KVT_STAGES slots, 1>  3 CTAs per SM; a warp owns accumulators w
+//                                   and w + 4 and alternates between them, so
+//                                   consecutive tiles of a warp are independent
+//   <4 warps, 3 slots, 1>           2 CTAs per SM
+//   <8 warps, 3 slots, 1>           1 CTA per SM: one accumulator per warp,
+//                                   twice the warps per SM
+//   <8 / kSub warps, 6 or 8 slots, kSub>
+//                                   a split shared by kSub = 2, 4 or 8 CTAs,
+//                                   one accumulator per warp: grids that
+//                                   would leave SMs without work
 constexpr int kAccs = 8;
 // Lazy softmax maximum: the reference moves when a logit exceeds it by more
 // than this many powers of two (P then stays at most 2^8 = 256).
@@ -62,14 +69,12 @@ constexpr float kLazyLog2 = 8.f;
 #ifndef KVT_WAVE_MARGIN
 #define KVT_WAVE_MARGIN 0.1   // last-wave fill gain that moves a grid to 2 CTAs per SM
 #endif
-constexpr int kWarpsNarrow = 4, kWarpsWide = 8;
+constexpr int kWarpsNarrow = 4;
 constexpr int kStagesFull = KVT_STAGES;    // 3 CTAs per SM
 constexpr int kStagesHalf = 3;             // 2 CTAs per SM
-constexpr int kStagesOne = 3;              // 1 CTA per SM (8 warps)
 __host__ __device__ constexpr int decode_smem(int warps, int stages) {
     return warps * stages * kTileBytes + 1024 + 256;   // rings, alignment, barriers
 }
-static_assert(kWarpsWide * kStagesOne * 8 <= 256, "mbarriers must fit their 256-byte area");
 static_assert(kWarpsNarrow * kStagesHalf * 8 <= 256, "mbarriers must fit their 256-byte area");
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s
 
@@ -97,6 +102,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// Non-blocking form: has the phase completed?
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(bar), "r"(parity)
@@ -142,8 +160,7 @@ __device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t &r0, uint32_t 
 // D = A(16x16 bf16, row) * B(16x8 bf16, col) + D, fp32 accumulate.
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                          uint32_t a3, uint32_t b0, uint32_t b1) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
         "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
@@ -196,14 +213,40 @@ __device__ __forceinline__ float fold(float x, float c, float w, float y) {
 __device__ __forceinline__ void lse_step(float &m, float &lsum, float4 &acc, const float2 v,
                                          const float4 o) {
     const float mn = fmaxf(m, v.x);
-    const float c = ex2(m - mn);                   // rescale what is summed so far
-    const float w = ex2(v.x - mn);
+    const float ref = mn == -INFINITY ? 0.f : mn;  // two empty states stay (-inf, 0, 0)
+    const float c = ex2(m - ref);                  // rescale what is summed so far
+    const float w = ex2(v.x - ref);
     m = mn;
     lsum = fold(lsum, c, w, v.y);
     acc.x = fold(acc.x, c, w, o.x);
     acc.y = fold(acc.y, c, w, o.y);
     acc.z = fold(acc.z, c, w, o.z);
     acc.w = fold(acc.w, c, w, o.w);
+}
+
+// kN states merged as a tree of neighbours; the result is in place 0.
+template <int kN>
+__device__ __forceinline__ void lse_tree(float (&m)[kN], float (&l)[kN], float4 (&acc)[kN]) {
+#pragma unroll
+    for (int w = 1; w < kN; w *= 2) {
+#pragma unroll
+        for (int v = 0; v + w < kN; v += 2 * w)
+            lse_step(m[v], l[v], acc[v], make_float2(m[v + w], l[v + w]), acc[v + w]);
+    }
+}
+
+// Dims 4*lane .. 4*lane + 3 of output row `row`.
+__device__ __forceinline__ void store_out(const DecodeArgs &a, int64_t row, int lane,
+                                          const float4 y) {
+    if (a.out_bf16) {
+        float r0, r1;
+        uint2 pk;
+        pk.x = pack_bf16(y.x, y.y, r0, r1);
+        pk.y = pack_bf16(y.z, y.w, r0, r1);
+        reinterpret_cast<uint2 *>(reinterpret_cast<uint16_t *>(a.out) + row * kHeadDim)[lane] = pk;
+    } else {
+        reinterpret_cast<float4 *>(a.out + row * kHeadDim)[lane] = y;
+    }
 }
 
 // The chains' states merged in chain order and normalised; lane t writes
@@ -227,38 +270,30 @@ __device__ __forceinline__ void merge_chains_store(const DecodeArgs &a, int64_t 
         lt = __fmaf_rn(c, l[q], lt);
     }
     const float inv = __frcp_rn(lt);
-    const float4 y = make_float4(__fmul_rn(r.x, inv), __fmul_rn(r.y, inv), __fmul_rn(r.z, inv),
-                                 __fmul_rn(r.w, inv));
-    if (a.out_bf16) {
-        float r0, r1;
-        uint2 pk;
-        pk.x = pack_bf16(y.x, y.y, r0, r1);
-        pk.y = pack_bf16(y.z, y.w, r0, r1);
-        reinterpret_cast<uint2 *>(reinterpret_cast<uint16_t *>(a.out) + row * kHeadDim)[lane] = pk;
-    } else {
-        reinterpret_cast<float4 *>(a.out + row * kHeadDim)[lane] = y;
-    }
+    store_out(a, row, lane, make_float4(__fmul_rn(r.x, inv), __fmul_rn(r.y, inv),
+                                        __fmul_rn(r.z, inv), __fmul_rn(r.w, inv)));
 }
 
-// The merge of one query head's ns (2..16) split partials by one warp. Every
+// The merge of one query head's ns (2 .. 4 * kPer) split partials by one warp. Every
 // load is issued before the first is used (indices clamped into the row, so
 // the loads need no guard): lane t loads split t's (m, l), shared by shuffle,
 // and each lane its 4 dims of every split's accumulator. The partials come
 // from L2 (.cg), written there by other SMs.
+template <int kPer>   // splits per chain, at most
 __device__ __forceinline__ void merge_head_regs(const DecodeArgs &a, int64_t row, int ns,
-                                                     int lane) {
+                                                int lane) {
     const int64_t base = row * a.max_splits;
     const float2 mine = __ldcg(reinterpret_cast<const float2 *>(a.part_ml) + base +
                                min(lane, ns - 1));
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o + base * kHeadDim) + lane;
-    float4 o[kMergeChains][4];
+    float4 o[kMergeChains][kPer];
     int s0[kMergeChains], n[kMergeChains];
 #pragma unroll
     for (int q = 0; q < kMergeChains; ++q) {
         s0[q] = (q * ns) / kMergeChains;
         n[q] = ((q + 1) * ns) / kMergeChains - s0[q];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) o[q][i] = __ldcg(po + min(s0[q] + i, ns - 1) * (kHeadDim / 4));
+        for (int i = 0; i < kPer; ++i) o[q][i] = __ldcg(po + min(s0[q] + i, ns - 1) * (kHeadDim / 4));
     }
     float m[kMergeChains], l[kMergeChains];
     float4 acc[kMergeChains];
@@ -268,7 +303,7 @@ __device__ __forceinline__ void merge_head_regs(const DecodeArgs &a, int64_t row
         l[q] = 0.f;
         acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < kPer; ++i) {
             const int sp = min(s0[q] + i, ns - 1);
             const float2 v = make_float2(__shfl_sync(0xffffffffu, mine.x, sp),
                                          __shfl_sync(0xffffffffu, mine.y, sp));
@@ -278,19 +313,130 @@ __device__ __forceinline__ void merge_head_regs(const DecodeArgs &a, int64_t row
     merge_chains_store(a, row, lane, m, l, acc);
 }
 
+// Q^T fragments (mma B operand): head n = lane/4 of the group, dims
+// 16*ks + 2*(lane%4) + {0,1} and +8. `row0` is the group's first q row.
+__device__ __forceinline__ void load_q(const DecodeArgs &a, int64_t row0, int G, int lane,
+                                       uint32_t (&qb)[8][2]) {
+    const int n = lane >> 2;
+    const bool live = n < G;
+    const uint32_t *qrow = reinterpret_cast<const uint32_t *>(a.q + (row0 + (live ? n : 0)) *
+                                                                        kHeadDim) + (lane & 3);
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) {
+        qb[ks][0] = live ? qrow[ks * 8] : 0u;
+        qb[ks][1] = live ? qrow[ks * 8 + 4] : 0u;
+    }
+}
+
+// Offset of a lane's ldmatrix row in a tile, for 16-dim step i of K (A operand
+// of S^T, row = token) and of V (A operand of O^T, loaded transposed, row =
+// token). Steps i and i + 4 lie one half apart.
+__device__ __forceinline__ uint32_t k_offset(int lane, int i) {
+    return (i >> 2) * kHalfBytes + swz((lane & 7) + ((lane >> 3) & 1) * 8, 2 * (i & 3) + (lane >> 4));
+}
+__device__ __forceinline__ uint32_t v_offset(int lane, int i) {
+    return (2 + (i >> 2)) * kHalfBytes + swz((lane & 7) + (lane >> 4) * 8, 2 * (i & 3) + ((lane >> 3) & 1));
+}
+
+// The session's last tile, in `slot` (one warp). Fused append: token T-1
+// arrives with this call; its K and V rows replace whatever the copy brought
+// for that slot and are stored to the reserved pool slot (lanes 0-15 move K,
+// 16-31 V, 16 B each). Slots past T may hold anything (NaN); P is 0 there but
+// 0 * NaN is not, so their V rows are cleared.
+__device__ __forceinline__ void finish_tail(const DecodeArgs &a, const int32_t *trow, int T,
+                                            int tok_base, int l, int lb, int g, uint8_t *slot,
+                                            int lane) {
+    const Shape &sh = a.s;
+    if (a.k_new != nullptr) {
+        const int r = T - 1 - tok_base;
+        const int u = lane & 15;
+        const int isv = lane >> 4;
+        const uint4 val = *reinterpret_cast<const uint4 *>(
+            (isv ? a.v_new : a.k_new) + (static_cast<int64_t>(lb) * sh.Hkv + g) * kHeadDim + u * 8);
+        *reinterpret_cast<uint4 *>(slot + isv * 2 * kHalfBytes + (u >> 3) * kHalfBytes +
+                                   swz(r, u & 7)) = val;
+        const int j = (T - 1) / sh.bt;
+        const int blk = trow[j];
+        if (blk >= 0 && blk < sh.num_blocks) {   // a bad id was flagged by the copy
+            const int row = ((blk * sh.L + l) * 2 * sh.Hkv + g) * sh.bt + (T - 1 - j * sh.bt) +
+                            isv * sh.Hkv * sh.bt;   // the pool has fewer than 2^31 rows
+            *reinterpret_cast<uint4 *>(a.hot + static_cast<int64_t>(row) * kHeadDim + u * 8) = val;
+        }
+    }
+    const int first_bad = T - tok_base;
+    const int units = (kTileTokens - first_bad) * 16;
+#pragma unroll 1
+    for (int u = lane; u < units; u += 32)
+        *reinterpret_cast<uint4 *>(slot + 2 * kHalfBytes + ((u >> 3) & 1) * kHalfBytes +
+                                   (first_bad + (u >> 4)) * 128 + (u & 7) * 16) =
+            make_uint4(0u, 0u, 0u, 0u);
+    // The slot is refilled by the async proxy later.
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+}
+
+constexpr int kOStride = kHeadDim + 4;   // floats per head row of a state in shared memory (bank skew)
+constexpr int kAccFloats = kMaxGroup * kOStride + 2 * kMaxGroup;   // O rows, m[8], l[8]
+
+// The CTA's kHere accumulator states (state(v), in shared memory) merged as a
+// tree of neighbours: a CTA that holds a part of a split's accumulators has a
+// node of the whole split's tree. One warp per head, four dims per lane, so a
+// warp reads one head's row of a state as 32 consecutive float4. A session of
+// one split held by one CTA is finished here; others leave a partial.
+template <int kHere, int kSub, int kWarps, typename State>
+__device__ __forceinline__ void merge_states(const DecodeArgs &a, int64_t row_base, int G,
+                                             int nsplit, int split, int sub, State state) {
+    const int lane = threadIdx.x & 31;
+    const int d0 = lane * 4;
+#pragma unroll 1
+    for (int h = threadIdx.x >> 5; h < G; h += kWarps) {
+        float m[kHere], l[kHere];
+        float4 acc[kHere];
+#pragma unroll
+        for (int v = 0; v < kHere; ++v) {
+            const float *ws = state(v);
+            m[v] = ws[kMaxGroup * kOStride + h];
+            l[v] = ws[kMaxGroup * kOStride + kMaxGroup + h];
+            acc[v] = *reinterpret_cast<const float4 *>(ws + h * kOStride + d0);
+        }
+        lse_tree<kHere>(m, l, acc);
+        if (kSub == 1 && nsplit == 1) {
+            const float inv = __frcp_rn(l[0]);
+            store_out(a, row_base + h, lane,
+                      make_float4(__fmul_rn(acc[0].x, inv), __fmul_rn(acc[0].y, inv),
+                                  __fmul_rn(acc[0].z, inv), __fmul_rn(acc[0].w, inv)));
+        } else {
+            const int64_t prow = ((row_base + h) * a.max_splits + split) * kSub + sub;
+            *reinterpret_cast<float4 *>(a.part_o + prow * kHeadDim + d0) = acc[0];
+            if (lane == 0)
+                *reinterpret_cast<float2 *>(a.part_ml + prow * 2) = make_float2(m[0], l[0]);
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
-// K1: one CTA = (split s, kv-head g, layer-batch row lb = li*B + b).
+// K1: kSub CTAs = (split s, kv-head g, layer-batch row lb = li*B + b).
 // The split's tiles go round robin to kAccs = 8 accumulators; warp w of the
-// kWarps consumes tiles w, w + kWarps, ... through its own ring of kStages
-// 8 KiB slots, tile k of the warp feeding its accumulator k % (8 / kWarps).
+// split's kStep = kWarps * kSub consumes tiles w, w + kStep, ... through its
+// own ring of kStages 8 KiB slots, tile k of the warp feeding its accumulator
+// k % (8 / kStep).
 // Per tile (16 tokens):
 //   S^T[16 tok x 8 heads] = K[16 x 128] . Q^T       8 x mma m16n8k16
 //   online softmax over tokens (columns = heads)
 //   O^T[128 x 8] += V^T[128 x 16] . P^T[16 x 8]     8 x mma, P^T via movmatrix
-// The accumulators merge in shared memory in accumulator order; a one-split
-// session writes its normalised output, others write (m, l, acc) partials,
+// The CTA's accumulators merge in shared memory; a one-split session held by
+// one CTA writes its normalised output, others write (m, l, acc) partials,
 // which the group's last CTA to finish merges when the launch allows it
-// (a.merge_max_splits), else the combine kernel.
+// (a.merge_max_splits), else a combine kernel.
+//
+// Large grids are bound by HBM. A small one (a layer of one or a few
+// sessions) is a chain of latencies: the previous call's end, q, a warp's
+// tiles one after another (0.36 us each; 0.16 us in a batch of 4, whose 64
+// mma.sync alone take 0.27 us of one tensor pipe), the merge, the combine.
+// It also runs every instruction once or twice, so its code has to stay in
+// the instruction cache (straight-line code of over about 32 KB is fetched at
+// 2.7 cycles an instruction): loops that are not on the tile path stay rolled
+// and the rare steps are in one place.
 // ---------------------------------------------------------------------------
 struct AccState {
     float m0, m1;   // running max, heads 2(lane%4) and +1 (log2 units)
@@ -298,11 +444,13 @@ struct AccState {
     float o[8][4];  // O^T fragments
 };
 
-template <int kWarps, int kStages>
+template <int kWarps, int kStages, int kSub>
 __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages == kStagesFull ? 3 : 1)
     decode_split_kernel(const __grid_constant__ CUtensorMap map, const DecodeArgs a) {
-    constexpr int kA = kAccs / kWarps;   // accumulators per warp
-    static_assert(kA * kWarps == kAccs, "accumulators divide among the warps");
+    constexpr int kStep = kWarps * kSub;  // warps of the split's CTAs
+    constexpr int kA = kAccs / kStep;     // accumulators per warp
+    static_assert(kA * kStep == kAccs, "accumulators divide among the warps");
+    static_assert(kA == 1 || (kA == 2 && kSub == 1), "two accumulators only in an unshared split");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -312,16 +460,19 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     // read here head-fastest so the CTAs of one split's kv-heads, whose runs
     // sit side by side in each block, start together (measured slightly
     // faster than split-fastest; the work of each CTA is the same).
-    const int64_t lin = blockIdx.x + static_cast<int64_t>(gridDim.x) *
-                                         (blockIdx.y + static_cast<int64_t>(gridDim.y) * blockIdx.z);
-    const int g = static_cast<int>(lin % gridDim.y);
-    const int split = static_cast<int>((lin / gridDim.y) % gridDim.x);
-    const int lb = static_cast<int>(lin / (static_cast<int64_t>(gridDim.y) * gridDim.x));
+    const uint32_t lin = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
+    const uint32_t run = lin / gridDim.y;
+    const int g = static_cast<int>(lin - run * gridDim.y);
+    const int slice = static_cast<int>(run % gridDim.x);
+    const int split = slice / kSub;
+    const int sub = slice % kSub;           // which of the split's CTAs
+    const int lb = static_cast<int>(run / gridDim.x);
     const int b = lb % a.B;
     const int li = lb / a.B;
     const int l = a.layer0 + li;
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
+    const int first = sub * kWarps + warp;  // this warp's first tile of the split
     const Shape sh = a.s;
     const int G = sh.Hq / sh.Hkv;
 
@@ -335,16 +486,16 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     // known before T: their block ids load alongside T instead of after it.
     // Lanes past the session's tiles may read table entries past its blocks
     // (never used).
-    constexpr int kMinWarpTiles = KVT_SPLIT_MIN_TILES / kWarps;
+    constexpr int kMinWarpTiles = KVT_SPLIT_MIN_TILES / kStep;
     const bool fixed_split = split_tiles(a.max_blocks * sh.bt) == KVT_SPLIT_MIN_TILES;
     int early_blk = 0;
     if (fixed_split && lane < kMinWarpTiles) {
-        const int j = (split * KVT_SPLIT_MIN_TILES + warp + lane * kWarps) * kTileTokens / sh.bt;
+        const int j = (split * KVT_SPLIT_MIN_TILES + first + lane * kStep) * kTileTokens / sh.bt;
         if (j < a.max_blocks) early_blk = trow[j];
     }
     const int T = a.seq_lens[b];
     if (T < 1 || T > a.max_blocks * sh.bt) {
-        if (split == 0 && g == 0 && threadIdx.x == 0) atomicOr(a.err, kErrBadLength);
+        if (slice == 0 && g == 0 && threadIdx.x == 0) atomicOr(a.err, kErrBadLength);
         return;
     }
     const int nsplit = num_splits(T);
@@ -352,22 +503,21 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     const int st = split_tiles(T);
     const int tile0 = split * st;
     const int tile1 = min(tiles_of(T), tile0 + st);
-    const int my_tiles = (tile1 - tile0 - warp + kWarps - 1) / kWarps;  // may be <= 0
+    const int my_tiles = (tile1 - tile0 - first + kStep - 1) / kStep;  // may be <= 0
 
     uint8_t *ring = smem + warp * kStages * kTileBytes;
     const uint32_t ring_s = smem_u32(ring);
     const uint32_t bar0 = smem_u32(bars + warp * kStages);
-    const int chunk_rows = sh.Hkv * sh.bt;   // rows between K and V runs
 
     // Block ids of this warp's tiles, fetched together up front: lane t
     // holds the block of the warp's tile t, so no table load waits in front
     // of a tile copy (one CTA per SM has no other warps to hide it behind).
-    static_assert((KVT_SPLIT_MAX_TILES + kWarps - 1) / kWarps <= 32,
+    static_assert((KVT_SPLIT_MAX_TILES + kStep - 1) / kStep <= 32,
                   "a warp's tiles of one split must fit one block id per lane");
-    static_assert(KVT_SPLIT_MIN_TILES % kWarps == 0, "whole tiles per warp");
+    static_assert(KVT_SPLIT_MIN_TILES % kStep == 0, "whole tiles per warp");
     int lane_blk = early_blk;
     if (!fixed_split && lane < my_tiles)
-        lane_blk = trow[(tile0 + warp + lane * kWarps) * kTileTokens / sh.bt];
+        lane_blk = trow[(tile0 + first + lane * kStep) * kTileTokens / sh.bt];
 
     if (lane == 0) {
         for (int i = 0; i < kStages; ++i) mbar_init(bar0 + 8 * i, 1);
@@ -378,7 +528,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     // Producer step (lane 0): tile k of this warp, in block blk, into slot
     // k % kStages.
     auto issue = [&](int k, int blk) {
-        const int ti = tile0 + warp + k * kWarps;
+        const int ti = tile0 + first + k * kStep;
         const int tok = ti * kTileTokens;
         const int j = tok / sh.bt;
         if (blk < 0 || blk >= sh.num_blocks) {
@@ -390,16 +540,16 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
         const uint32_t bar = bar0 + 8 * (k % kStages);
         // inject_extra_tx (a test of the bounded wait, 0 in normal calls): this
         // one barrier then never completes its phase, although every copy lands.
-        const bool injected = k == 0 && warp == 0 && split == 0 && g == 0 && lb == 0;
+        const bool injected = k == 0 && warp == 0 && slice == 0 && g == 0 && lb == 0;
         mbar_expect_tx(bar, kTileBytes + (injected ? a.inject_extra_tx : 0));
         tma_load_tile(slot, &map, rowk, bar);
     };
     // The block of tile k, for every lane (k < 32 wherever it is used).
     auto blk_of = [&](int k) { return __shfl_sync(0xffffffffu, lane_blk, k & 31); };
-#pragma unroll
-    for (int k = 0; k < kStages; ++k) {
+#pragma unroll 1
+    for (int k = 0; k < kStages && k < my_tiles; ++k) {
         const int blk = blk_of(k);
-        if (lane == 0 && k < my_tiles) issue(k, blk);
+        if (lane == 0) issue(k, blk);
     }
 
     // Everything above reads only the hot pool, the block table and seq_lens.
@@ -411,18 +561,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     // Q^T fragments (mma B operand): head n = lane/4 of the group, dims
     // 16*ks + 2*(lane%4) + {0,1} and +8.
     uint32_t qb[8][2];
-    {
-        const int n = lane >> 2;
-        const bool live = n < G;
-        const uint32_t *qrow = reinterpret_cast<const uint32_t *>(
-            a.q + ((static_cast<int64_t>(li) * a.B + b) * sh.Hq + g * G + (live ? n : 0)) *
-                      kHeadDim);
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            qb[ks][0] = live ? qrow[ks * 8 + (lane & 3)] : 0u;
-            qb[ks][1] = live ? qrow[ks * 8 + 4 + (lane & 3)] : 0u;
-        }
-    }
+    load_q(a, static_cast<int64_t>(lb) * sh.Hq + g * G, G, lane, qb);
 
     AccState acc_state[kA];
 #pragma unroll
@@ -436,43 +575,24 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     const float sl = a.scale_log2;
     int fail_k = -1;
 
-    // ldmatrix lane roles. K (A operand, row-major): row = token.
-    const int krow = (lane & 7) + ((lane >> 3) & 1) * 8;
-    const int khi = lane >> 4;
-    // V (A operand of O^T, loaded transposed): row = token.
-    const int vrow = (lane & 7) + (lane >> 4) * 8;
-    const int vhi = (lane >> 3) & 1;
+    uint32_t koff[4], voff[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        koff[j] = k_offset(lane, j);
+        voff[j] = v_offset(lane, j);
+    }
 
-    // Fused append: token T-1 arrives with this call. Its K and V rows
-    // replace whatever the copy brought for that slot of tile k and are
-    // stored to the reserved pool slot. Lanes 0-15 move K, 16-31 V, 16 B each.
-    auto splice_new = [&](int k, int tok_base) {
-        const int r = T - 1 - tok_base;
-        const int u = lane & 15;
-        const int isv = lane >> 4;
-        const uint4 val = *reinterpret_cast<const uint4 *>(
-            (isv ? a.v_new : a.k_new) +
-            ((static_cast<int64_t>(li) * a.B + b) * sh.Hkv + g) * kHeadDim + u * 8);
-        *reinterpret_cast<uint4 *>(ring + (k % kStages) * kTileBytes + isv * 2 * kHalfBytes +
-                                   (u >> 3) * kHalfBytes + swz(r, u & 7)) = val;
-        const int j = (T - 1) / sh.bt;
-        const int blk = trow[j];
-        if (blk >= 0 && blk < sh.num_blocks) {   // a bad id was flagged by the copy
-            const int64_t row =
-                ((static_cast<int64_t>(blk) * sh.L + l) * 2 * sh.Hkv + g) * sh.bt +
-                (T - 1 - j * sh.bt) + isv * chunk_rows;
-            *reinterpret_cast<uint4 *>(a.hot + row * kHeadDim + u * 8) = val;
-        }
-        // The slot is refilled by the async proxy later.
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncwarp();
+    auto load_k = [&](uint32_t slot, int ks, uint32_t (&f)[4]) {
+        ldsm_x4(slot + koff[ks & 3] + (ks >> 2) * kHalfBytes, f[0], f[1], f[2], f[3]);
+    };
+    auto load_values = [&](uint32_t slot, uint32_t (&f)[8][4]) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            ldsm_x4_t(slot + voff[i & 3] + (i >> 2) * kHalfBytes, f[i][0], f[i][1], f[i][2], f[i][3]);
     };
     // One k-step (16 dims) of S^T = K . Q^T into acc.
-    auto qk_step = [&](uint32_t slot, int ks, float (&acc)[4]) {
-        uint32_t r0, r1, r2, r3;
-        const int u = 2 * ks + khi;
-        ldsm_x4(slot + (u >> 3) * kHalfBytes + swz(krow, u & 7), r0, r1, r2, r3);
-        mma_bf16(acc, r0, r1, r2, r3, qb[ks][0], qb[ks][1]);
+    auto qk_step = [&](const uint32_t (&f)[4], int ks, float (&acc)[4]) {
+        mma_bf16(acc, f[0], f[1], f[2], f[3], qb[ks][0], qb[ks][1]);
     };
     // Logits in log2 units; tokens at or past T are -inf.
     auto logits = [&](const float (&sa)[4], const float (&sb)[4], int tok_base, float (&x)[4]) {
@@ -483,108 +603,192 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
         x[2] = v1 ? (sa[2] + sb[2]) * sl : -INFINITY;
         x[3] = v1 ? (sa[3] + sb[3]) * sl : -INFINITY;
     };
-    // Last, partial tile: slots past T may hold anything (NaN); P is 0 there
-    // but 0 * NaN is not, so clear those V rows of tile k.
-    auto clear_tail_v = [&](int k, int tok_base) {
-        if (tok_base + kTileTokens > T) {
-            const int first_bad = T - tok_base;
-            const int units = (kTileTokens - first_bad) * 16;
-            uint8_t *vp = ring + (k % kStages) * kTileBytes + 2 * kHalfBytes;
-            for (int u = lane; u < units; u += 32) {
-                const int r = first_bad + (u >> 4);
-                const int h = (u >> 3) & 1;
-                *reinterpret_cast<uint4 *>(vp + h * kHalfBytes + r * 128 + (u & 7) * 16) =
-                    make_uint4(0u, 0u, 0u, 0u);
-            }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
+    auto tile_base = [&](int k) { return (tile0 + first + k * kStep) * kTileTokens; };
+
+    // Online-softmax step with a lazy maximum: the reference point m moves
+    // only when a logit of the tile exceeds it by more than kLazyLog2 (the
+    // first tile always does, m starting at -inf); otherwise P = 2^(x - m)
+    // stays at most 2^kLazyLog2 and neither m, l nor the accumulator are
+    // rescaled. When it moves, m becomes the exact running maximum (a
+    // quad-shuffle reduction over the tile's columns) and l and O are
+    // rescaled by 2^(m_old - m_new). The decision is the warp's and depends
+    // only on the tile's logits and the state, so every launch variant takes
+    // it alike.
+    auto grows = [&](const float (&x)[4], const AccState &s) {
+        return (x[0] > s.m0 + kLazyLog2) | (x[2] > s.m0 + kLazyLog2) |
+               (x[1] > s.m1 + kLazyLog2) | (x[3] > s.m1 + kLazyLog2);
+    };
+    auto move_max = [&](const float (&x)[4], AccState &s) {
+        float mx0 = fmaxf(x[0], x[2]), mx1 = fmaxf(x[1], x[3]);
+#pragma unroll
+        for (int off = 4; off < 32; off <<= 1) {
+            mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, off));
+            mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, off));
+        }
+        const float mn0 = fmaxf(s.m0, mx0), mn1 = fmaxf(s.m1, mx1);
+        const float al0 = ex2(s.m0 - mn0), al1 = ex2(s.m1 - mn1);
+        s.m0 = mn0;
+        s.m1 = mn1;
+        s.l0 *= al0;
+        s.l1 *= al1;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            s.o[i][0] *= al0;
+            s.o[i][1] *= al1;
+            s.o[i][2] *= al0;
+            s.o[i][3] *= al1;
         }
     };
-    auto tile_base = [&](int k) { return (tile0 + warp + k * kWarps) * kTileTokens; };
-
-    // One tile into accumulator s: scores, softmax, O^T += V^T . P^T.
-    // False: its wait timed out.
-    auto one_tile = [&](int k, AccState &s) -> bool {
-        const uint32_t slot = ring_s + (k % kStages) * kTileBytes;
-        if (!mbar_wait(bar0 + 8 * (k % kStages), (k / kStages) & 1)) return false;
-        const int tok_base = tile_base(k);
-        if (a.k_new != nullptr && tok_base + kTileTokens >= T) splice_new(k, tok_base);
-
-        // S^T = K . Q^T, two accumulators to shorten the mma chain.
-        float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int ks = 0; ks < 8; ks += 2) {
-            qk_step(slot, ks, sa);
-            qk_step(slot, ks + 1, sb);
-        }
-        float x[4];
-        logits(sa, sb, tok_base, x);
-        // Online-softmax step with a lazy maximum: the reference point m moves
-        // only when a logit of the tile exceeds it by more than kLazyLog2 (the
-        // first tile always does, m starting at -inf); otherwise P = 2^(x - m)
-        // stays at most 2^kLazyLog2 and neither m, l nor the accumulator are
-        // rescaled. When it moves, m becomes the exact running maximum (a
-        // quad-shuffle reduction over the tile's columns) and l and O are
-        // rescaled by 2^(m_old - m_new). P is rounded to bf16, as the PV
-        // product sees it. The decision is the warp's and depends only on the
-        // tile's logits and the state, so every launch variant takes it alike.
-        const bool grow = (x[0] > s.m0 + kLazyLog2) | (x[2] > s.m0 + kLazyLog2) |
-                          (x[1] > s.m1 + kLazyLog2) | (x[3] > s.m1 + kLazyLog2);
-        if (__any_sync(0xffffffffu, grow)) {
-            float mx0 = fmaxf(x[0], x[2]), mx1 = fmaxf(x[1], x[3]);
-#pragma unroll
-            for (int off = 4; off < 32; off <<= 1) {
-                mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, off));
-                mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, off));
-            }
-            const float mn0 = fmaxf(s.m0, mx0), mn1 = fmaxf(s.m1, mx1);
-            const float al0 = ex2(s.m0 - mn0), al1 = ex2(s.m1 - mn1);
-            s.m0 = mn0;
-            s.m1 = mn1;
-            s.l0 *= al0;
-            s.l1 *= al1;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                s.o[i][0] *= al0;
-                s.o[i][1] *= al1;
-                s.o[i][2] *= al0;
-                s.o[i][3] *= al1;
-            }
-        }
+    // P of a tile (rounded to bf16, as the PV product sees it) as the PV
+    // product's B fragment; its rounded values join the normaliser.
+    auto weights = [&](const float (&x)[4], AccState &s, uint32_t &pb0, uint32_t &pb1) {
         float q0, q1, q2, q3;
         const uint32_t p01 = pack_bf16(ex2(x[0] - s.m0), ex2(x[1] - s.m1), q0, q1);
         const uint32_t p23 = pack_bf16(ex2(x[2] - s.m0), ex2(x[3] - s.m1), q2, q3);
         s.l0 += q0 + q2;
         s.l1 += q1 + q3;
-        const uint32_t pb0 = movmatrix_t(p01);   // P^T tokens 0-7  -> B fragment
-        const uint32_t pb1 = movmatrix_t(p23);   // P^T tokens 8-15
-        clear_tail_v(k, tok_base);
-        const uint32_t vslot = slot + 2 * kHalfBytes;
+        pb0 = movmatrix_t(p01);   // P^T tokens 0-7  -> B fragment
+        pb1 = movmatrix_t(p23);   // P^T tokens 8-15
+    };
+    // O^T += V^T . P^T
+    auto add_values = [&](const uint32_t (&f)[8][4], AccState &s, uint32_t pb0, uint32_t pb1) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            uint32_t r0, r1, r2, r3;
-            const int u = 2 * i + vhi;
-            ldsm_x4_t(vslot + (u >> 3) * kHalfBytes + swz(vrow, u & 7), r0, r1, r2, r3);
-            mma_bf16(s.o[i], r0, r1, r2, r3, pb0, pb1);
-        }
-        __syncwarp();
+        for (int i = 0; i < 8; ++i) mma_bf16(s.o[i], f[i][0], f[i][1], f[i][2], f[i][3], pb0, pb1);
+    };
+    auto slot_of = [&](int k) { return ring_s + (k % kStages) * kTileBytes; };
+    auto refill = [&](int k) {
+        if (k + kStages >= my_tiles) return;
         const int nblk = blk_of(k + kStages);
-        if (lane == 0 && k + kStages < my_tiles) issue(k + kStages, nblk);
+        if (lane == 0) issue(k + kStages, nblk);
+    };
+
+    // One tile into accumulator s. False: its wait timed out.
+    auto one_tile = [&](int k, AccState &s) -> bool {
+        if (!mbar_wait(bar0 + 8 * (k % kStages), (k / kStages) & 1)) return false;
+        const int tok_base = tile_base(k);
+        const uint32_t slot = slot_of(k);
+        if (tok_base + kTileTokens >= T)
+            finish_tail(a, trow, T, tok_base, l, lb, g, ring + (k % kStages) * kTileBytes, lane);
+        // S^T = K . Q^T, two accumulators to shorten the mma chain.
+        float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f}, x[4];
+        uint32_t kf[8][4], vf[8][4];
+#pragma unroll
+        for (int ks = 0; ks < 8; ++ks) load_k(slot, ks, kf[ks]);
+#pragma unroll
+        for (int ks = 0; ks < 8; ks += 2) {
+            qk_step(kf[ks], ks, sa);
+            qk_step(kf[ks + 1], ks + 1, sb);
+        }
+        // A warp with one accumulator has the registers to bring V in while
+        // the softmax runs.
+        if constexpr (kA == 1) load_values(slot, vf);
+        logits(sa, sb, tok_base, x);
+        if (__any_sync(0xffffffffu, grows(x, s))) move_max(x, s);
+        uint32_t pb0, pb1;
+        weights(x, s, pb0, pb1);
+        if constexpr (kA == 2) load_values(slot, vf);
+        add_values(vf, s, pb0, pb1);
+        __syncwarp();
+        refill(k);
         return true;
     };
 
-    // Consecutive tiles of a warp feed different accumulators (kA = 2), so
-    // the second tile's work does not wait for the first tile's products.
-    for (int k = 0; k < my_tiles; k += kA) {
-        if (!one_tile(k, acc_state[0])) {
-            fail_k = k;
-            break;
+    // kN consecutive tiles that have all landed, none of them the session's
+    // last, into the one accumulator of a warp: the values of one_tile on each
+    // in turn, with the score products side by side and the next fragments on
+    // their way while a step's products run. The weights follow together too,
+    // unless a tile after the first of all moves the maximum: then nothing has
+    // been added yet and the caller takes the tiles one by one (false).
+    auto tile_batch = [&](auto n_const, int k, AccState &s) -> bool {
+        constexpr int kN = decltype(n_const)::value;
+        float sa[kN][4], sb[kN][4], x[kN][4];
+#pragma unroll
+        for (int i = 0; i < kN; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) sa[i][j] = sb[i][j] = 0.f;
+        uint32_t f[2][2 * kN][4];
+        auto load_step = [&](int ks) {
+#pragma unroll
+            for (int i = 0; i < kN; ++i) {
+                load_k(slot_of(k + i), ks, f[(ks >> 1) & 1][2 * i]);
+                load_k(slot_of(k + i), ks + 1, f[(ks >> 1) & 1][2 * i + 1]);
+            }
+        };
+        load_step(0);
+#pragma unroll
+        for (int ks = 0; ks < 8; ks += 2) {
+            if (ks + 2 < 8) load_step(ks + 2);
+#pragma unroll
+            for (int i = 0; i < kN; ++i) {
+                qk_step(f[(ks >> 1) & 1][2 * i], ks, sa[i]);
+                qk_step(f[(ks >> 1) & 1][2 * i + 1], ks + 1, sb[i]);
+            }
         }
-        if constexpr (kA == 2) {
+        uint32_t vf[2][8][4];
+        load_values(slot_of(k), vf[0]);
+#pragma unroll
+        for (int i = 0; i < kN; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[i][j] = (sa[i][j] + sb[i][j]) * sl;
+        if (k == 0 && __any_sync(0xffffffffu, grows(x[0], s))) move_max(x[0], s);
+        bool grow = false;
+#pragma unroll
+        for (int i = 0; i < kN; ++i) grow |= grows(x[i], s);
+        if (__any_sync(0xffffffffu, grow)) return false;
+        uint32_t pb[kN][2];
+#pragma unroll
+        for (int i = 0; i < kN; ++i) weights(x[i], s, pb[i][0], pb[i][1]);
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+            if (i + 1 < kN) load_values(slot_of(k + i + 1), vf[(i + 1) & 1]);
+            add_values(vf[i & 1], s, pb[i][0], pb[i][1]);
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int i = 0; i < kN; ++i) refill(k + i);
+        return true;
+    };
+
+    if constexpr (kA == 2) {
+        // Consecutive tiles of a warp feed different accumulators, so the
+        // second tile's work does not wait for the first tile's products.
+#pragma unroll 1
+        for (int k = 0; k < my_tiles; k += 2) {
+            if (!one_tile(k, acc_state[0])) {
+                fail_k = k;
+                break;
+            }
             if (k + 1 < my_tiles && !one_tile(k + 1, acc_state[1])) {
                 fail_k = k + 1;
                 break;
             }
+        }
+    } else {
+        constexpr int kBatch = kStages >= 4 ? 4 : 2;
+        // The warp's tiles before the session's last one need no length mask.
+        const int plain = tile_base(my_tiles - 1) + kTileTokens >= T ? my_tiles - 1 : my_tiles;
+        int single = 0;   // tiles up to here go one by one
+#pragma unroll 1
+        for (int k = 0; k < my_tiles;) {
+            bool batch = k >= single && k + kBatch <= plain;
+            if (batch) {
+#pragma unroll
+                for (int i = 0; i < kBatch; ++i)
+                    batch &= mbar_test(bar0 + 8 * ((k + i) % kStages), ((k + i) / kStages) & 1);
+                batch = __all_sync(0xffffffffu, batch);
+            }
+            if (batch) {
+                if (tile_batch(std::integral_constant<int, kBatch>{}, k, acc_state[0])) {
+                    k += kBatch;
+                    continue;
+                }
+                single = k + kBatch;
+            }
+            if (!one_tile(k, acc_state[0])) {
+                fail_k = k;
+                break;
+            }
+            ++k;
         }
     }
 
@@ -592,6 +796,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
         if (lane == 0) atomicOr(a.err, kErrTimeout);
         // Tiles fail_k .. fail_k+kStages-1 were issued and not consumed: wait
         // (again bounded) for them so no copy lands after the CTA exits.
+#pragma unroll 1
         for (int k = fail_k; k < fail_k + kStages && k < my_tiles; ++k)
             mbar_wait(bar0 + 8 * (k % kStages), (k / kStages) & 1);
     }
@@ -599,8 +804,6 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     // Accumulator states -> this warp's own ring (all of its loads have
     // completed): accumulator v = warp + kWarps * i at float offset
     // i * kAccFloats of warp (v % kWarps)'s ring.
-    constexpr int kOStride = kHeadDim + 4;   // floats per head row (bank skew)
-    constexpr int kAccFloats = kMaxGroup * kOStride + 2 * kMaxGroup;   // O rows, m[8], l[8]
     static_assert(kA * kAccFloats * 4 <= kStages * kTileBytes, "states fit the ring");
 #pragma unroll
     for (int i = 0; i < kA; ++i) {
@@ -631,55 +834,13 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     }
     __syncthreads();
 
-    // Merge the accumulators in order; a thread handles (head, 4 dims), so a
-    // warp reads one head's row of each state as 32 consecutive float4.
-    auto acc_base = [&](int v) {
-        return reinterpret_cast<const float *>(smem + (v % kWarps) * kStages * kTileBytes) +
-               (v / kWarps) * kAccFloats;
-    };
     const int64_t row_base = static_cast<int64_t>(lb) * sh.Hq + g * G;
-    for (int e = threadIdx.x; e < G * (kHeadDim / 4); e += blockDim.x) {
-        const int h = e / (kHeadDim / 4);
-        const int d0 = (e % (kHeadDim / 4)) * 4;
-        float M = -INFINITY;
-#pragma unroll
-        for (int v = 0; v < kAccs; ++v) M = fmaxf(M, acc_base(v)[kMaxGroup * kOStride + h]);
-        float lsum = 0.f;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int v = 0; v < kAccs; ++v) {
-            const float *wsv = acc_base(v);
-            const float *wmv = wsv + kMaxGroup * kOStride;
-            const float sc = ex2(wmv[h] - M);      // an accumulator with no tile: m = -inf, 0
-            lsum += sc * wmv[8 + h];
-            const float4 x = *reinterpret_cast<const float4 *>(wsv + h * kOStride + d0);
-            acc.x += sc * x.x;
-            acc.y += sc * x.y;
-            acc.z += sc * x.z;
-            acc.w += sc * x.w;
-        }
-        if (nsplit == 1) {
-            const float inv = 1.f / lsum;
-            if (a.out_bf16) {
-                uint2 pk;
-                float r0, r1;
-                pk.x = pack_bf16(acc.x * inv, acc.y * inv, r0, r1);
-                pk.y = pack_bf16(acc.z * inv, acc.w * inv, r0, r1);
-                *reinterpret_cast<uint2 *>(reinterpret_cast<uint16_t *>(a.out) +
-                                           (row_base + h) * kHeadDim + d0) = pk;
-            } else {
-                *reinterpret_cast<float4 *>(a.out + (row_base + h) * kHeadDim + d0) =
-                    make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
-            }
-        } else {
-            const int64_t prow = (row_base + h) * a.max_splits + split;
-            *reinterpret_cast<float4 *>(a.part_o + prow * kHeadDim + d0) = acc;
-            if (d0 == 0) {
-                a.part_ml[prow * 2] = M;
-                a.part_ml[prow * 2 + 1] = lsum;
-            }
-        }
-    }
+    merge_states<kAccs / kSub, kSub, kWarps>(
+        a, row_base, G, nsplit, split, sub, [&](int v) {
+            return reinterpret_cast<const float *>(smem + (v % kWarps) * kStages * kTileBytes) +
+                   (v / kWarps) * kAccFloats;
+        });
+    if (kWarps != kWarpsNarrow || kSub > 1) return;
     if (nsplit == 1 || nsplit > a.merge_max_splits) return;
 
     // Arrival. Every split of the group arrives once, whatever happened in
@@ -697,7 +858,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     __syncthreads();
     if (!s_last) return;
 #pragma unroll 1
-    for (int h = warp; h < G; h += kWarps) merge_head_regs(a, row_base + h, nsplit, lane);
+    for (int h = warp; h < G; h += kWarps) merge_head_regs<kSplitKernelMerge / kMergeChains>(a, row_base + h, nsplit, lane);
 }
 
 // K2 for tables of at most kRegMergeMax splits: one warp per (layer-batch
@@ -715,7 +876,7 @@ __global__ void __launch_bounds__(128) decode_combine_small_kernel(const DecodeA
     const int ns = num_splits(T);
     if (ns <= 1 || ns <= a.merge_max_splits) return;   // written by K1
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    merge_head_regs(a, row, ns, threadIdx.x & 31);
+    merge_head_regs<kRegMergeMax / kMergeChains>(a, row, ns, threadIdx.x & 31);
 }
 
 // K2 for wider tables: one CTA (4 warps) per (layer-batch row, q-head) of a
@@ -784,6 +945,79 @@ __global__ void __launch_bounds__(128) decode_combine_kernel(const DecodeArgs a)
     }
 }
 
+// K2 for splits shared by kSub CTAs (small grids, at most kRegMergeMax
+// splits): one CTA of four warps per (layer-batch row, q-head). Warp w loads
+// every partial of chain w at once (at most four splits, kSub states each),
+// joins each split's states as the split kernel joins accumulators, and folds
+// the chain; warp 0 merges the chains. Latency-bound: one round trip to L2,
+// then 0.4 us of dependent steps. A warp per split, with the chains folded
+// from shared memory, took 0.5 us longer.
+template <int kSub>
+__global__ void __launch_bounds__(128) decode_combine_sub_kernel(const DecodeArgs a) {
+    asm volatile("griddepcontrol.launch_dependents;");   // a following overlapped call
+    const int64_t row = blockIdx.x;                // lb * Hq + h
+    const int b = static_cast<int>((row / a.s.Hq) % a.B);
+    const int T = a.seq_lens[b];                   // before the wait, as K1 reads it
+    if (T < 1 || T > a.max_blocks * a.s.bt) return;
+    const int ns = num_splits(T);
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const int s0 = (warp * ns) / kMergeChains;
+    const int n = ((warp + 1) * ns) / kMergeChains - s0;
+    const int64_t base = row * a.max_splits * kSub;
+    const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + base;
+    const float4 *po = reinterpret_cast<const float4 *>(a.part_o + base * kHeadDim) + lane;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __shared__ float s_m[kMergeChains], s_l[kMergeChains];
+    __shared__ float4 s_acc[kMergeChains][kHeadDim / 4];
+    constexpr int kPer = kRegMergeMax / kMergeChains;
+    float2 v[kPer][kSub];
+    float4 o[kPer][kSub];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        if (i < n) {
+#pragma unroll
+            for (int r = 0; r < kSub; ++r) {
+                const int p = (s0 + i) * kSub + r;
+                v[i][r] = __ldcg(ml + p);
+                o[i][r] = __ldcg(po + p * (kHeadDim / 4));
+            }
+        }
+    }
+    float m = -INFINITY, lsum = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        if (i < n) {
+            float mr[kSub], lr[kSub];
+#pragma unroll
+            for (int r = 0; r < kSub; ++r) {
+                mr[r] = v[i][r].x;
+                lr[r] = v[i][r].y;
+            }
+            lse_tree<kSub>(mr, lr, o[i]);
+            lse_step(m, lsum, acc, make_float2(mr[0], lr[0]), o[i][0]);
+        }
+    }
+    s_acc[warp][lane] = acc;
+    if (lane == 0) {
+        s_m[warp] = m;
+        s_l[warp] = lsum;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        float mq[kMergeChains], lq[kMergeChains];
+        float4 aq[kMergeChains];
+#pragma unroll
+        for (int q = 0; q < kMergeChains; ++q) {
+            mq[q] = s_m[q];
+            lq[q] = s_l[q];
+            aq[q] = s_acc[q][lane];
+        }
+        merge_chains_store(a, row, lane, mq, lq, aq);
+    }
+}
+
 }  // namespace
 
 bool encode_hot_tensor_map(CUtensorMap *map, void *hot_base, int64_t rows, int64_t run_rows,
@@ -823,19 +1057,29 @@ bool encode_hot_tensor_map(CUtensorMap *map, void *hot_base, int64_t rows, int64
     return true;
 }
 
+template <int kWarps, int kStages, int kSub>
+static cudaError_t prepare_split() {
+    return cudaFuncSetAttribute(decode_split_kernel<kWarps, kStages, kSub>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                decode_smem(kWarps, kStages));
+}
+
 cudaError_t prepare_kernels() {
-    cudaError_t e = cudaFuncSetAttribute(decode_split_kernel<kWarpsNarrow, kStagesFull>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         decode_smem(kWarpsNarrow, kStagesFull));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(decode_split_kernel<kWarpsNarrow, kStagesHalf>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 decode_smem(kWarpsNarrow, kStagesHalf));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(decode_split_kernel<kWarpsWide, kStagesOne>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 decode_smem(kWarpsWide, kStagesOne));
+    cudaError_t e = prepare_split<kWarpsNarrow, kStagesFull, 1>();
+    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1>();
+    if (e == cudaSuccess) e = prepare_split<8, 3, 1>();
+    if (e == cudaSuccess) e = prepare_split<4, 6, 2>();
+    if (e == cudaSuccess) e = prepare_split<2, 6, 4>();
+    if (e == cudaSuccess) e = prepare_split<1, 8, 8>();
     return e;
+}
+
+template <int kWarps, int kStages, int kSub>
+static cudaError_t launch_split(cudaLaunchConfig_t &c, const CUtensorMap &map, const DecodeArgs &a) {
+    c.gridDim.x *= kSub;
+    c.blockDim = dim3(kWarps * 32);
+    c.dynamicSmemBytes = decode_smem(kWarps, kStages);
+    return cudaLaunchKernelEx(&c, decode_split_kernel<kWarps, kStages, kSub>, map, a);
 }
 
 cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_sms,
@@ -871,24 +1115,41 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // the combine: 256 x 4K-token sessions per layer +1.3 %, 8 x 4K all
     // layers +1.6 %; one 4K- or 16K-token session per layer -7 % / -5 % and
     // 32 x 4K -5 % when shorter grids merged too).
+    // Grids that would leave SMs idle: each split is shared by as many CTAs as
+    // still get an SM of their own. A CTA then has fewer bytes to draw through
+    // its SM (a 64-tile split is 512 KB, 6 us for one SM), holds more of them
+    // in its ring before the previous call ends, and its warps no longer share
+    // tensor pipes; the combine reads kSub states per split instead of one.
+    // One session per layer in us per layer, unshared and shared: 1K tokens
+    // 6.25 and 5.10, 3 001 8.04 and 5.36, 8K 8.51 and 6.74, 16 391 9.97 and
+    // 8.72; 4 sessions of 1 280 8.26 and 6.17. Two CTAs per SM (rings half as
+    // deep) were slower: 8K 8.17, 16 391 10.6. Tables of over kRegMergeMax
+    // splits have long splits and over 64 CTAs per kv-head group already, and
+    // a caller's scratch may have no room for the extra rows.
+    int sub = 1;
+    if (splits <= kRegMergeMax)
+        while (sub < 8 && 2 * sub * ctas <= static_cast<int64_t>(num_sms) &&
+               2 * sub * static_cast<int64_t>(splits) * a.s.Hq * a.nlayers * a.B <= a.part_rows)
+            sub *= 2;
     DecodeArgs ka = a;
     ka.merge_max_splits = ctas >= 8 * static_cast<int64_t>(num_sms) ? kSplitKernelMerge : 0;
     cudaError_t e;
-    if (ctas <= num_sms) {
-        c1.blockDim = dim3(kWarpsWide * 32);
-        c1.dynamicSmemBytes = decode_smem(kWarpsWide, kStagesOne);
-        e = cudaLaunchKernelEx(&c1, decode_split_kernel<kWarpsWide, kStagesOne>, map, ka);
-    } else if (ctas <= 2 * static_cast<int64_t>(num_sms) || fill(2) > fill(3) + KVT_WAVE_MARGIN) {
-        c1.dynamicSmemBytes = decode_smem(kWarpsNarrow, kStagesHalf);
-        e = cudaLaunchKernelEx(&c1, decode_split_kernel<kWarpsNarrow, kStagesHalf>, map, ka);
-    } else {
-        c1.dynamicSmemBytes = decode_smem(kWarpsNarrow, kStagesFull);
-        e = cudaLaunchKernelEx(&c1, decode_split_kernel<kWarpsNarrow, kStagesFull>, map, ka);
-    }
+    if (sub == 8)
+        e = launch_split<1, 8, 8>(c1, map, ka);
+    else if (sub == 4)
+        e = launch_split<2, 6, 4>(c1, map, ka);
+    else if (sub == 2)
+        e = launch_split<4, 6, 2>(c1, map, ka);
+    else if (ctas <= num_sms)
+        e = launch_split<8, 3, 1>(c1, map, ka);
+    else if (ctas <= 2 * static_cast<int64_t>(num_sms) || fill(2) > fill(3) + KVT_WAVE_MARGIN)
+        e = launch_split<kWarpsNarrow, kStagesHalf, 1>(c1, map, ka);
+    else
+        e = launch_split<kWarpsNarrow, kStagesFull, 1>(c1, map, ka);
     if (e != cudaSuccess) return e;
     // Every session's output written by the split kernel: one split each, or
     // few enough splits to merge there.
-    if (splits <= 1 || splits <= ka.merge_max_splits) return cudaSuccess;
+    if (sub == 1 && (splits <= 1 || splits <= ka.merge_max_splits)) return cudaSuccess;
 
     const int64_t rows = static_cast<int64_t>(a.nlayers) * a.B * a.s.Hq;
     cudaLaunchConfig_t c2 = {};
@@ -897,6 +1158,12 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     c2.stream = st;
     c2.attrs = attr;
     c2.numAttrs = 1;
+    if (sub > 1) {
+        c2.gridDim = dim3(static_cast<unsigned>(rows));
+        if (sub == 2) return cudaLaunchKernelEx(&c2, decode_combine_sub_kernel<2>, ka);
+        if (sub == 4) return cudaLaunchKernelEx(&c2, decode_combine_sub_kernel<4>, ka);
+        return cudaLaunchKernelEx(&c2, decode_combine_sub_kernel<8>, ka);
+    }
     if (splits <= kRegMergeMax) {
         c2.gridDim = dim3(static_cast<unsigned>((rows + 3) / 4));
         return cudaLaunchKernelEx(&c2, decode_combine_small_kernel, ka);

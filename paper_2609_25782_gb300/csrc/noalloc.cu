@@ -180,8 +180,11 @@ extern "C" int decode_attention_noalloc(const kv_pool_config *cfg, int32_t layer
     a.tables = block_tables;
     a.seq_lens = seq_lens;
     a.out = out;
+    // The partials' two arrays over the whole scratch: the check above leaves
+    // room for prow rows, small grids may use more of them.
+    a.part_rows = (KV_NOALLOC_SCRATCH_BYTES - 256) / ((kvt::kHeadDim + 2) * 4);
     a.part_o = reinterpret_cast<float *>(scratch);
-    a.part_ml = reinterpret_cast<float *>(scratch + o_bytes);
+    a.part_ml = reinterpret_cast<float *>(scratch + a.part_rows * kvt::kHeadDim * 4);
     a.counters = counters;
     a.err = flag;
     a.B = B;

@@ -105,6 +105,7 @@ struct kv_pool {
     int32_t table_stride = 0;            // max blocks per session
     int32_t max_splits = 0;              // split bound for max_context
     int64_t part_rows = 0;               // decode workspace capacity (partial rows)
+    int64_t part_alloc = 0;              // partial rows allocated (at least part_rows)
     int num_sms = 1;
     int mig_ctas = 0;                    // cap on migration-kernel CTAs, 0 = none
     kvt::Shape shape{};
@@ -458,7 +459,10 @@ int kv_pool_create(const kv_pool_config *cfg, kv_pool **out) {
             return bail(fail(KV_ERR_CUDA, "cudaSetDevice failed"));
         cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, c.device);
         const int64_t tbl = static_cast<int64_t>(c.max_sessions) * p->table_stride * 4;
-        const int64_t prow = p->part_rows;
+        // Small grids share a split among CTAs, each writing its own partial
+        // row: at most one CTA per SM, eight heads each, beyond part_rows.
+        p->part_alloc = std::max<int64_t>(p->part_rows, int64_t(p->num_sms) * kvt::kMaxGroup);
+        const int64_t prow = p->part_alloc;
         int rc = p->cuda("cudaMalloc(tables)", [&] { return cudaMalloc(&p->d_tables, tbl); });
         if (!rc) rc = p->cuda("cudaMalloc(partials)", [&] {
             return cudaMalloc(&p->d_part_o, prow * kvt::kHeadDim * sizeof(float));
@@ -467,7 +471,7 @@ int kv_pool_create(const kv_pool_config *cfg, kv_pool **out) {
             return cudaMalloc(&p->d_part_ml, prow * 2 * sizeof(float));
         });
         // A multi-split call has at most part_rows / Hq layer-batch rows.
-        p->counter_count = prow / c.num_q_heads * c.num_kv_heads;
+        p->counter_count = p->part_rows / c.num_q_heads * c.num_kv_heads;
         const int64_t cnt = p->counter_count * 4;
         if (!rc) rc = p->cuda("cudaMalloc(counters)", [&] { return cudaMalloc(&p->d_counters, cnt); });
         if (!rc) rc = p->cuda("cudaMemset", [&] { return cudaMemset(p->d_counters, 0, cnt); });
@@ -902,6 +906,7 @@ static int decode_impl(kv_pool *p, int32_t layer, const void *q, const void *k_n
     a.out = out;
     a.part_o = p->d_part_o;
     a.part_ml = p->d_part_ml;
+    a.part_rows = p->part_alloc;
     a.counters = p->d_counters;
     a.err = p->d_err;
     a.B = B;
