@@ -546,9 +546,12 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
     };
     // The block of tile k, for every lane (k < 32 wherever it is used).
     auto blk_of = [&](int k) { return __shfl_sync(0xffffffffu, lane_blk, k & 31); };
+    // a.pace > 0 (launch_decode): at most that many of the warp's tiles in
+    // flight while the previous kernel may still be running.
 #pragma unroll 1
     for (int k = 0; k < kStages && k < my_tiles; ++k) {
         const int blk = blk_of(k);
+        if (a.pace > 0 && k >= a.pace) mbar_wait(bar0 + 8 * (k - a.pace), 0);
         if (lane == 0) issue(k, blk);
     }
 
@@ -1132,6 +1135,17 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
                2 * sub * static_cast<int64_t>(splits) * a.s.Hq * a.nlayers * a.B <= a.part_rows)
             sub *= 2;
     DecodeArgs ka = a;
+    // An overlapped call whose CTAs are all resident at once fills its rings
+    // while the previous call still merges: 20-30 MB of copies queued in front
+    // of that call's partials, this call's q and the end of the grid between
+    // them. Paced to one tile per warp (two with four warps per SM), the copies
+    // still keep HBM busy and the chain behind them is shorter. us per layer,
+    // unpaced and paced: one session of 16 391 tokens 8.64 and 7.98, 32K 13.6
+    // and 12.7; 8 x 4K 15.0 and 13.2, 12 x 2K 12.1 and 11.4; 4 x 16K 24.1 and
+    // 23.1. Rings that cover a whole split (4 or 8 CTAs per split) showed no
+    // difference; in grids of more than one wave the later CTAs lose by it
+    // (8 x 16K 44.4 and 45.1).
+    ka.pace = !overlap_previous ? 0 : sub == 2 ? 2 : sub == 1 && ctas <= 2 * static_cast<int64_t>(num_sms) ? 1 : 0;
     ka.merge_max_splits = ctas >= 8 * static_cast<int64_t>(num_sms) ? kSplitKernelMerge : 0;
     cudaError_t e;
     if (sub == 8)
