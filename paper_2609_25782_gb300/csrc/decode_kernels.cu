@@ -8,13 +8,12 @@
 //                          In a long grid, the last CTA of a kv-head of a
 //                          session of at most 4 splits to finish merges them
 //                          (log-sum-exp in a fixed order).
-//   decode_combine_small_kernel, decode_combine_kernel
+//   decode_combine_small_kernel, decode_combine_kernel, decode_combine_shared_kernel
 //                          the same merge for the other multi-split sessions
 //                          (one warp per query head from registers, up to 16
-//                          splits; else four warps per head), launched as a
+//                          splits; four warps per head for more, and where
+//                          several CTAs shared a split), launched as a
 //                          programmatic dependent of the split kernel.
-//   decode_combine_sub_kernel
-//                          the same where several CTAs shared each split.
 //
 // Hot pool: hot[NB][L][2][Hkv][bt][128] bf16. A (block, layer, K|V, head)
 // run is bt rows of 256 B, row = ((blk*L + l)*2 + kv)*Hkv + g)*bt + slot. The
@@ -58,10 +57,9 @@ constexpr int kHalfBytes = 2048;           // 16 rows x 128 B (64 dims)
 //   <4 warps, 3 slots, 1>           2 CTAs per SM
 //   <8 warps, 3 slots, 1>           1 CTA per SM: one accumulator per warp,
 //                                   twice the warps per SM
-//   <8 / kSub warps, 6 or 8 slots, kSub>
-//                                   a split shared by kSub = 2, 4 or 8 CTAs,
-//                                   one accumulator per warp: grids that
-//                                   would leave SMs without work
+//   <8 / kSub warps, slots, kSub>   a split shared by kSub = 2, 4 or 8 CTAs,
+//                                   one accumulator per warp: grids of up to
+//                                   three CTAs per SM once shared
 constexpr int kAccs = 8;
 // Lazy softmax maximum: the reference moves when a logit exceeds it by more
 // than this many powers of two (P then stays at most 2^8 = 256).
@@ -358,20 +356,19 @@ __device__ __forceinline__ void finish_tail(const DecodeArgs &a, const int32_t *
         const int j = (T - 1) / sh.bt;
         const int blk = trow[j];
         if (blk >= 0 && blk < sh.num_blocks) {   // a bad id was flagged by the copy
-            const int row = ((blk * sh.L + l) * 2 * sh.Hkv + g) * sh.bt + (T - 1 - j * sh.bt) +
-                            isv * sh.Hkv * sh.bt;   // the pool has fewer than 2^31 rows
-            *reinterpret_cast<uint4 *>(a.hot + static_cast<int64_t>(row) * kHeadDim + u * 8) = val;
+            const int at = ((blk * sh.L + l) * 2 * sh.Hkv + g) * sh.bt + (T - 1 - j * sh.bt) +
+                           isv * sh.Hkv * sh.bt;   // the pool has fewer than 2^31 rows
+            *reinterpret_cast<uint4 *>(a.hot + static_cast<int64_t>(at) * kHeadDim + u * 8) = val;
         }
     }
-    const int first_bad = T - tok_base;
-    const int units = (kTileTokens - first_bad) * 16;
-#pragma unroll 1
-    for (int u = lane; u < units; u += 32)
-        *reinterpret_cast<uint4 *>(slot + 2 * kHalfBytes + ((u >> 3) & 1) * kHalfBytes +
-                                   (first_bad + (u >> 4)) * 128 + (u & 7) * 16) =
-            make_uint4(0u, 0u, 0u, 0u);
-    // The slot is refilled by the async proxy later.
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    const int row = T - tok_base + (lane >> 4);   // this lane's rows: row, row + 2, ...
+    uint8_t *vp = slot + (2 + ((lane >> 3) & 1)) * kHalfBytes + row * 128 + (lane & 7) * 16;
+#pragma unroll
+    for (int j = 0; j < kTileTokens / 2; ++j)
+        if (row + 2 * j < kTileTokens)
+            *reinterpret_cast<uint4 *>(vp + j * 256) = make_uint4(0u, 0u, 0u, 0u);
+    // No copy is issued into the slot after this (it is the warp's last tile),
+    // so its reads need no ordering against the async proxy.
     __syncwarp();
 }
 
@@ -445,7 +442,7 @@ struct AccState {
 };
 
 template <int kWarps, int kStages, int kSub>
-__global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages == kStagesFull ? 3 : 1)
+__global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kStages == 2 ? 3 : kStages == 3 ? 2 : 1)
     decode_split_kernel(const __grid_constant__ CUtensorMap map, const DecodeArgs a) {
     constexpr int kStep = kWarps * kSub;  // warps of the split's CTAs
     constexpr int kA = kAccs / kStep;     // accumulators per warp
@@ -682,14 +679,14 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
             qk_step(kf[ks], ks, sa);
             qk_step(kf[ks + 1], ks + 1, sb);
         }
-        // A warp with one accumulator has the registers to bring V in while
-        // the softmax runs.
-        if constexpr (kA == 1) load_values(slot, vf);
+        // The warps of a shared split have no others to hide behind: V comes in
+        // while the softmax runs.
+        if constexpr (kSub > 1) load_values(slot, vf);
         logits(sa, sb, tok_base, x);
         if (__any_sync(0xffffffffu, grows(x, s))) move_max(x, s);
         uint32_t pb0, pb1;
         weights(x, s, pb0, pb1);
-        if constexpr (kA == 2) load_values(slot, vf);
+        if constexpr (kSub == 1) load_values(slot, vf);
         add_values(vf, s, pb0, pb1);
         __syncwarp();
         refill(k);
@@ -763,6 +760,14 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps == kWarpsNarrow && kStages
             }
             if (k + 1 < my_tiles && !one_tile(k + 1, acc_state[1])) {
                 fail_k = k + 1;
+                break;
+            }
+        }
+    } else if constexpr (kSub == 1) {
+#pragma unroll 1
+        for (int k = 0; k < my_tiles; ++k) {
+            if (!one_tile(k, acc_state[0])) {
+                fail_k = k;
                 break;
             }
         }
@@ -883,12 +888,15 @@ __global__ void __launch_bounds__(128) decode_combine_small_kernel(const DecodeA
 }
 
 // K2 for wider tables: one CTA (4 warps) per (layer-batch row, q-head) of a
-// multi-split session the split kernel did not merge. Warp w folds chain w, the contiguous quarter
-// [w*ns/4, (w+1)*ns/4) of the splits (split order), then warp 0 merges the
-// four chains in order. The result depends only on the partials
-// and ns. Launched as a programmatic dependent of K1: it waits for K1's
-// completion with griddepcontrol.wait, so its CTAs can already be resident
-// while K1 drains.
+// multi-split session the split kernel did not merge. Warp w folds chain w, the
+// contiguous quarter [w*ns/4, (w+1)*ns/4) of the splits (split order), each
+// split's kSub states joined first as the split kernel joins accumulators, then
+// warp 0 merges the four chains in order. The result depends only on the
+// partials and ns. Launched as a programmatic dependent of K1: it waits for
+// K1's completion with griddepcontrol.wait, so its CTAs can already be resident
+// while K1 drains. Batches of kBatch splits: every load of a batch is issued
+// before the first is folded (indices clamped into the quarter, no guards).
+template <int kSub, int kBatch>
 __global__ void __launch_bounds__(128) decode_combine_kernel(const DecodeArgs a) {
     asm volatile("griddepcontrol.launch_dependents;");   // a following overlapped call
     const int64_t row = blockIdx.x;                // lb * Hq + h
@@ -899,35 +907,43 @@ __global__ void __launch_bounds__(128) decode_combine_kernel(const DecodeArgs a)
     const int T = a.seq_lens[b];
     if (T < 1 || T > a.max_blocks * a.s.bt) return;
     const int ns = num_splits(T);
-    if (ns <= 1 || ns <= a.merge_max_splits) return;   // written by K1
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (kSub == 1 && (ns <= 1 || ns <= a.merge_max_splits)) return;   // written by K1
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int64_t base = row * a.max_splits;
+    const int64_t base = row * a.max_splits * kSub;
     const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + base;
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o + base * kHeadDim) + lane;
     __shared__ float s_m[kCombineWarps], s_l[kCombineWarps];
     __shared__ float4 s_acc[kCombineWarps][kHeadDim / 4];
-
     const int s0 = (warp * ns) / kCombineWarps;
     const int s1 = ((warp + 1) * ns) / kCombineWarps;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     float m = -INFINITY, lsum = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    // Batches of kCombineBatch splits: every load of a batch is issued before
-    // the first is folded (indices clamped into the quarter, no guards).
-    constexpr int kCombineBatch = 16;
-    for (int sb = s0; sb < s1; sb += kCombineBatch) {
-        float2 v[kCombineBatch];
-        float4 o[kCombineBatch];
+#pragma unroll 1
+    for (int sb = s0; sb < s1; sb += kBatch) {
+        float2 v[kBatch][kSub];
+        float4 o[kBatch][kSub];
 #pragma unroll
-        for (int j = 0; j < kCombineBatch; ++j) {
-            const int sp = min(sb + j, s1 - 1);
-            v[j] = ml[sp];
-            o[j] = po[sp * (kHeadDim / 4)];
+        for (int j = 0; j < kBatch; ++j) {
+            const int sp = min(sb + j, s1 - 1) * kSub;
+#pragma unroll
+            for (int r = 0; r < kSub; ++r) {
+                v[j][r] = __ldcg(ml + sp + r);
+                o[j][r] = __ldcg(po + (sp + r) * (kHeadDim / 4));
+            }
         }
 #pragma unroll
-        for (int j = 0; j < kCombineBatch; ++j)
-            if (sb + j < s1) lse_step(m, lsum, acc, v[j], o[j]);
+        for (int j = 0; j < kBatch; ++j) {
+            float mr[kSub], lr[kSub];
+#pragma unroll
+            for (int r = 0; r < kSub; ++r) {
+                mr[r] = v[j][r].x;
+                lr[r] = v[j][r].y;
+            }
+            lse_tree<kSub>(mr, lr, o[j]);
+            if (sb + j < s1) lse_step(m, lsum, acc, make_float2(mr[0], lr[0]), o[j][0]);
+        }
     }
     s_acc[warp][lane] = acc;
     if (lane == 0) {
@@ -948,15 +964,15 @@ __global__ void __launch_bounds__(128) decode_combine_kernel(const DecodeArgs a)
     }
 }
 
-// K2 for splits shared by kSub CTAs (small grids, at most kRegMergeMax
-// splits): one CTA of four warps per (layer-batch row, q-head). Warp w loads
-// every partial of chain w at once (at most four splits, kSub states each),
-// joins each split's states as the split kernel joins accumulators, and folds
-// the chain; warp 0 merges the chains. Latency-bound: one round trip to L2,
-// then 0.4 us of dependent steps. A warp per split, with the chains folded
-// from shared memory, took 0.5 us longer.
+// K2 for splits shared by kSub CTAs, tables of at most kRegMergeMax splits: as
+// above, with all of a chain's partials (at most four splits of kSub states)
+// loaded at once. Latency-bound: one round trip to L2 (0.13 us, several times
+// that under the next call's copies), then 0.4 us of dependent steps. The loop
+// above in its place keeps fewer registers and starts its loads after each
+// other: 6.2 instead of 5.3 us per layer for one session of 3 001 tokens, 13.3
+// instead of 12.5 for 8 x 4K.
 template <int kSub>
-__global__ void __launch_bounds__(128) decode_combine_sub_kernel(const DecodeArgs a) {
+__global__ void __launch_bounds__(128) decode_combine_shared_kernel(const DecodeArgs a) {
     asm volatile("griddepcontrol.launch_dependents;");   // a following overlapped call
     const int64_t row = blockIdx.x;                // lb * Hq + h
     const int b = static_cast<int>((row / a.s.Hq) % a.B);
@@ -1072,6 +1088,8 @@ cudaError_t prepare_kernels() {
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1>();
     if (e == cudaSuccess) e = prepare_split<8, 3, 1>();
     if (e == cudaSuccess) e = prepare_split<4, 6, 2>();
+    if (e == cudaSuccess) e = prepare_split<4, 3, 2>();
+    if (e == cudaSuccess) e = prepare_split<4, 2, 2>();
     if (e == cudaSuccess) e = prepare_split<2, 6, 4>();
     if (e == cudaSuccess) e = prepare_split<1, 8, 8>();
     return e;
@@ -1109,31 +1127,47 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
         const double w = static_cast<double>(ctas) / (per_sm * static_cast<double>(num_sms));
         return w / static_cast<double>(static_cast<int64_t>(w) + (w > static_cast<int64_t>(w)));
     };
-    // Which sessions the split kernel merges itself (the bits are the same
-    // either way): those of up to kSplitKernelMerge splits, in grids of at
-    // least 8 CTAs per SM. There, many groups finish at different times and
-    // their merges spread over the grid. In shorter grids each CTA's arrival
-    // (an atomic round trip holding its SM slot) and the tail merges cost more
-    // than the combine launch (measured on GB300 against merging everything in
-    // the combine: 256 x 4K-token sessions per layer +1.3 %, 8 x 4K all
-    // layers +1.6 %; one 4K- or 16K-token session per layer -7 % / -5 % and
-    // 32 x 4K -5 % when shorter grids merged too).
-    // Grids that would leave SMs idle: each split is shared by as many CTAs as
-    // still get an SM of their own. A CTA then has fewer bytes to draw through
-    // its SM (a 64-tile split is 512 KB, 6 us for one SM), holds more of them
-    // in its ring before the previous call ends, and its warps no longer share
-    // tensor pipes; the combine reads kSub states per split instead of one.
-    // One session per layer in us per layer, unshared and shared: 1K tokens
-    // 6.25 and 5.10, 3 001 8.04 and 5.36, 8K 8.51 and 6.74, 16 391 9.97 and
-    // 8.72; 4 sessions of 1 280 8.26 and 6.17. Two CTAs per SM (rings half as
-    // deep) were slower: 8K 8.17, 16 391 10.6. Tables of over kRegMergeMax
-    // splits have long splits and over 64 CTAs per kv-head group already, and
-    // a caller's scratch may have no room for the extra rows.
+    // Splits shared by several CTAs. A grid of few CTAs leaves SMs idle, and
+    // each of its CTAs draws 512 KB or more through one SM (6 us) with its
+    // warps in each other's way; shared, a CTA has less to draw, holds more of
+    // it before the previous call ends, and is gone sooner, so the next call's
+    // CTAs start their copies sooner. The combine reads kSub states per split
+    // instead of one. us per layer, unshared and shared:
+    //   8 or 4 CTAs, at most one per SM: 1 x 3 001 8.04 and 5.36, 1 x 8K 8.51
+    //     and 6.74, 4 x 1 280 8.26 and 6.17
+    //   2, at most one per SM: 1 x 16 391 9.97 and 8.72 (two CTAs per SM with
+    //     half the ring 10.0, four of a shorter split 10.6)
+    //   2, two per SM: 8 x 4K 13.1 and 12.4, 2 x 16K 13.3 and 12.6, 5 x 5K 11.6
+    //     and 10.9 (three per SM 14.0, 14.0, 12.1)
+    //   2, three per SM: 8 x 5K 17.1 and 15.7, 10 x 4K 17.4 and 15.7, 3 x 16K
+    //     19.3 and 18.3; not the long splits of tables wider than 32K tokens
+    //     (1 x 100K 34.3 and 35.0), which do share at two per SM (1 x 40K 16.8
+    //     and 16.1)
+    // Sessions of one split need no combine unshared, and do not share: from a
+    // graph it would still pay for one to four of them above 512 tokens (1 x 1K
+    // 6.25 and 5.10, but 8 x 1K 6.98 and 6.94, 48 x 1 000 18.4 and 21.0), while
+    // direct calls would pay for the second launch. A caller's scratch may have
+    // no room for the extra rows.
+    const int64_t sms = num_sms;
+    const int64_t rows1 = static_cast<int64_t>(splits) * a.s.Hq * a.nlayers * a.B;
+    auto fits = [&](int sub, int per_sm) {
+        return sub * ctas <= per_sm * sms && sub * rows1 <= a.part_rows;
+    };
+    const bool wide = splits > kRegMergeMax;   // long splits, and a combine in batches
     int sub = 1;
-    if (splits <= kRegMergeMax)
-        while (sub < 8 && 2 * sub * ctas <= static_cast<int64_t>(num_sms) &&
-               2 * sub * static_cast<int64_t>(splits) * a.s.Hq * a.nlayers * a.B <= a.part_rows)
-            sub *= 2;
+    int per_sm = 1;   // of a shared grid
+    if (splits > 1) {
+        if (!wide && fits(8, 1))
+            sub = 8;
+        else if (!wide && fits(4, 1))
+            sub = 4;
+        else if (fits(2, 1))
+            sub = 2;
+        else if (fits(2, 2))
+            sub = per_sm = 2;
+        else if (!wide && fits(2, 3))
+            sub = 2, per_sm = 3;
+    }
     DecodeArgs ka = a;
     // An overlapped call whose CTAs are all resident at once fills its rings
     // while the previous call still merges: 20-30 MB of copies queued in front
@@ -1143,20 +1177,38 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // unpaced and paced: one session of 16 391 tokens 8.64 and 7.98, 32K 13.6
     // and 12.7; 8 x 4K 15.0 and 13.2, 12 x 2K 12.1 and 11.4; 4 x 16K 24.1 and
     // 23.1. Rings that cover a whole split (4 or 8 CTAs per split) showed no
-    // difference; in grids of more than one wave the later CTAs lose by it
-    // (8 x 16K 44.4 and 45.1).
-    ka.pace = !overlap_previous ? 0 : sub == 2 ? 2 : sub == 1 && ctas <= 2 * static_cast<int64_t>(num_sms) ? 1 : 0;
-    ka.merge_max_splits = ctas >= 8 * static_cast<int64_t>(num_sms) ? kSplitKernelMerge : 0;
+    // difference, and in grids of more than one wave the later CTAs lose by it
+    // (8 x 16K 44.4 and 45.1); unshared long splits take no part (1 x 100K).
+    ka.pace = 0;
+    if (overlap_previous && sub == 2)
+        ka.pace = per_sm == 1 ? 2 : 1;
+    else if (overlap_previous && sub == 1 && !wide && ctas <= 2 * sms)
+        ka.pace = 1;
+
+    // Which sessions the split kernel merges itself (the bits are the same
+    // either way): those of up to kSplitKernelMerge splits, in grids of at
+    // least 8 CTAs per SM. There, many groups finish at different times and
+    // their merges spread over the grid. In shorter grids each CTA's arrival
+    // (an atomic round trip holding its SM slot) and the tail merges cost more
+    // than the combine launch (measured on GB300 against merging everything in
+    // the combine: 256 x 4K-token sessions per layer +1.3 %, 8 x 4K all
+    // layers +1.6 %; one 4K- or 16K-token session per layer -7 % / -5 % and
+    // 32 x 4K -5 % when shorter grids merged too).
+    ka.merge_max_splits = ctas >= 8 * sms ? kSplitKernelMerge : 0;
     cudaError_t e;
     if (sub == 8)
         e = launch_split<1, 8, 8>(c1, map, ka);
     else if (sub == 4)
         e = launch_split<2, 6, 4>(c1, map, ka);
-    else if (sub == 2)
+    else if (sub == 2 && per_sm == 1)
         e = launch_split<4, 6, 2>(c1, map, ka);
-    else if (ctas <= num_sms)
+    else if (sub == 2 && per_sm == 2)
+        e = launch_split<4, 3, 2>(c1, map, ka);
+    else if (sub == 2)
+        e = launch_split<4, 2, 2>(c1, map, ka);
+    else if (ctas <= sms)
         e = launch_split<8, 3, 1>(c1, map, ka);
-    else if (ctas <= 2 * static_cast<int64_t>(num_sms) || fill(2) > fill(3) + KVT_WAVE_MARGIN)
+    else if (ctas <= 2 * sms || fill(2) > fill(3) + KVT_WAVE_MARGIN)
         e = launch_split<kWarpsNarrow, kStagesHalf, 1>(c1, map, ka);
     else
         e = launch_split<kWarpsNarrow, kStagesFull, 1>(c1, map, ka);
@@ -1172,18 +1224,17 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     c2.stream = st;
     c2.attrs = attr;
     c2.numAttrs = 1;
-    if (sub > 1) {
-        c2.gridDim = dim3(static_cast<unsigned>(rows));
-        if (sub == 2) return cudaLaunchKernelEx(&c2, decode_combine_sub_kernel<2>, ka);
-        if (sub == 4) return cudaLaunchKernelEx(&c2, decode_combine_sub_kernel<4>, ka);
-        return cudaLaunchKernelEx(&c2, decode_combine_sub_kernel<8>, ka);
-    }
-    if (splits <= kRegMergeMax) {
+    if (sub == 1 && !wide) {
         c2.gridDim = dim3(static_cast<unsigned>((rows + 3) / 4));
         return cudaLaunchKernelEx(&c2, decode_combine_small_kernel, ka);
     }
     c2.gridDim = dim3(static_cast<unsigned>(rows));
-    return cudaLaunchKernelEx(&c2, decode_combine_kernel, ka);
+    if (wide)
+        return sub == 2 ? cudaLaunchKernelEx(&c2, decode_combine_kernel<2, 8>, ka)
+                        : cudaLaunchKernelEx(&c2, decode_combine_kernel<1, 16>, ka);
+    if (sub == 8) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<8>, ka);
+    if (sub == 4) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<4>, ka);
+    return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<2>, ka);
 }
 
 }  // namespace kvt

@@ -20,33 +20,45 @@ from test_gpu_parity import TOL, direct_case, gpu_decode, host_hot, pkg, scaled_
 pytestmark = pytest.mark.gpu
 
 
-def ctas(lens, bt=16, Hkv=4):
-    """CTAs of the unshared grid: splits for the table width x kv-heads x rows."""
-    from paper_2609_25782_gb300 import kvtier
-    return kvtier.kv_decode_splits(-(-max(lens) // bt) * bt) * Hkv * len(lens)
+# (lengths of one call, table width in tokens, KV heads, CTAs that share a split
+# on a GPU of 152 SMs)
+CASES = [
+    ([1024], 1024, 4, 1), ([900] * 8, 1024, 4, 1),
+    ([1], 1040, 4, 8), ([16], 2048, 4, 8), ([17], 2048, 4, 8), ([127], 2048, 4, 8),
+    ([129], 2048, 4, 8), ([1024], 2048, 4, 8), ([1025], 2048, 4, 8), ([2047], 2048, 4, 8),
+    ([4096], 4096, 4, 8), ([4097], 5120, 4, 4), ([8193], 8704, 4, 4),
+    ([9300], 9728, 4, 2), ([16384], 16384, 4, 2), ([16391], 16448, 4, 2), ([19000], 19008, 4, 2),
+    ([2048, 1, 1025, 700], 2048, 4, 4), ([33, 1023, 15, 1040], 1088, 4, 4),
+    ([3000, 2049] * 2, 3072, 4, 2),
+    # two and three CTAs per SM
+    ([2500, 4096, 15, 1024] * 2, 4096, 4, 2), ([4096, 1, 3000, 17, 2048] * 2, 4096, 4, 2),
+    # tables of more than 16 splits; a chain of more splits than one batch of loads (35 splits)
+    ([40000], 40000, 4, 2), ([70001], 70016, 4, 2), ([33000, 500], 33024, 4, 2),
+    ([37000], 37120, 1, 2), ([40000, 36000], 40000, 1, 2),
+]
 
 
-# (lengths of one call, CTAs that share a split on a GPU of 128 to 159 SMs)
-@pytest.mark.parametrize("lens,shared", [
-    ([1], 8), ([16], 8), ([17], 8), ([127], 8), ([129], 8), ([1024], 8), ([1025], 8),
-    ([4096], 8), ([4097], 4), ([8192], 4), ([8193], 4), ([9300], 2), ([16384], 2), ([16391], 2), ([19000], 2),
-    ([1024] * 8, 4), ([2048, 1, 1025, 700], 4), ([33, 1023, 15, 1040], 4), ([3000, 2049] * 2, 2),
-])
+@pytest.mark.parametrize("lens,tokens,hkv,shared", CASES)
 @pytest.mark.parametrize("bt,scale", [(16, 1 / math.sqrt(128)), (64, 0.5)])
-def test_shared_splits(pkg, lens, shared, bt, scale):  # noqa: F811
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
-    if 128 <= sms < 160:
-        assert shared * ctas(lens, bt) <= sms and (shared == 8 or 2 * shared * ctas(lens, bt) > sms)
+def test_shared_splits(pkg, lens, tokens, hkv, shared, bt, scale):  # noqa: F811
+    from paper_2609_25782_gb300 import kvtier
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        ctas = kvtier.kv_decode_splits(-(-tokens // bt) * bt) * hkv * len(lens)
+        room = 3 * 152 if shared == 2 else 152
+        assert shared * ctas <= room
+        assert shared in (1, 8) or 2 * shared * ctas > 152 or tokens > 32768
     n = len(lens)
-    many = lens + [100] * (160 // n)            # a batch with at least 160 CTAs shares nothing
-    pool, sess, tables, q = direct_case(pkg, many, L=1, bt=bt, seed=17, max_batch=len(many))
+    many = lens + [100] * (520 // (n * hkv))    # a batch too large to share
+    pool, sess, tables, q = direct_case(pkg, many, L=1, Hq=8 * hkv, Hkv=hkv, bt=bt, seed=17,
+                                        max_batch=len(many))
     pool._scale = scale                         # 0.5: logits of std 5.7, so the maximum moves late
-    width = -(-max(lens) // bt)
-    got = gpu_decode(pool, 0, q[:, :n], tables[:n, :width].copy(), lens)[0]
+    width = -(-tokens // bt)
+    wide = np.pad(tables, ((0, 0), (0, max(0, width - tables.shape[1]))), constant_values=-1)
+    got = gpu_decode(pool, 0, q[:, :n], wide[:n, :width].copy(), lens)[0]
     whole = gpu_decode(pool, 0, q, tables, many)[0]
     assert np.array_equal(got.view(np.int64), whole[:n].view(np.int64))
     hot = host_hot(pool, 17, sess, many, tables)
     ref = oracle.paged_decode(hot, q[:, :n].cpu().view(torch.int16).numpy().view(np.uint16),
-                              tables[:n], lens, scale, 32)
+                              tables[:n], lens, scale, 8 * hkv)
     assert scaled_err(got, ref[0]) <= TOL
     assert pool.check_device() == 0
