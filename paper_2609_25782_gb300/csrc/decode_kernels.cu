@@ -48,7 +48,7 @@ constexpr int kTileBytes = 8192;           // K 4 KiB + V 4 KiB
 constexpr int kHalfBytes = 2048;           // 16 rows x 128 B (64 dims)
 // The plan of one split: its tiles are dealt round robin to kAccs running
 // softmax states (accumulator v takes tiles v, v + kAccs, ...), which merge
-// as a tree of neighbours (0 1, 2 3, ...; then pairs of pairs) at the end.
+// at the end, first each half of them, then the halves (join_accs).
 // That plan fixes the result; how the accumulators map to warps and CTAs is a
 // launch choice, and every choice gives bit-identical results:
 //   <4 warps, KVT_STAGES slots, 1>  3 CTAs per SM; a warp owns accumulators w
@@ -130,14 +130,30 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     return true;
 }
 
+// L2 policy of the K and V copies: each byte is read once per step, so its
+// line is the first to leave. Otherwise a layer's stream (over three times the
+// L2 for 32 sessions of 20K tokens) also pushes out the partials, which the
+// combine then reads from HBM behind the next call's copies: us per layer with
+// the default policy and this one, 16 x 14K tokens 72.7 and 70.2, 32 x 20K 191
+// and 185.5, 64 x 8K 154.3 and 150.4, 8 x 16K 45.2 and 44.1; sessions whose
+// layer fits the L2 the same. Calls that leave no partials for a combine keep
+// the default (256 x 1 000 81.1 and 82.0).
+__device__ __forceinline__ uint64_t copy_policy(bool stream) {
+    uint64_t p, q;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(q));
+    return stream ? p : q;
+}
+
 // One tile: the box (64 columns, 16 rows, 2 column halves, K and V) of the
 // hot pool's 4-D view, starting at K row `row`.
 __device__ __forceinline__ void tma_load_tile(uint32_t dst, const CUtensorMap *map, int row,
-                                              uint32_t bar) {
+                                              uint32_t bar, uint64_t policy) {
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(0), "r"(0), "r"(bar)
+        ".L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(0), "r"(0), "r"(bar),
+        "l"(policy)
         : "memory");
 }
 
@@ -222,15 +238,42 @@ __device__ __forceinline__ void lse_step(float &m, float &lsum, float4 &acc, con
     acc.w = fold(acc.w, c, w, o.w);
 }
 
-// kN states merged as a tree of neighbours; the result is in place 0.
+// The merge of a split's accumulators: each half (0-3 and 4-7) by its largest
+// maximum, then the two halves. kN = 8 is a whole split, 4 a half, 2 the two
+// halves; the result is in place 0. (Pairs, then pairs of pairs, would suit
+// every way of sharing, but its three levels cost a one-split call 0.1-0.2 us.)
 template <int kN>
-__device__ __forceinline__ void lse_tree(float (&m)[kN], float (&l)[kN], float4 (&acc)[kN]) {
+__device__ __forceinline__ void join_accs(float (&m)[kN], float (&l)[kN], float4 (&acc)[kN]) {
+    static_assert(kN == 1 || kN == 2 || kN == 4 || kN == 8, "parts of a split");
+    if constexpr (kN >= 4) {
 #pragma unroll
-    for (int w = 1; w < kN; w *= 2) {
+        for (int h = 0; h < kN; h += 4) {
+            const float mx = fmaxf(fmaxf(m[h], m[h + 1]), fmaxf(m[h + 2], m[h + 3]));
+            const float ref = mx == -INFINITY ? 0.f : mx;   // empty states stay (-inf, 0, 0)
+            float lsum = 0.f;
+            float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int v = 0; v + w < kN; v += 2 * w)
-            lse_step(m[v], l[v], acc[v], make_float2(m[v + w], l[v + w]), acc[v + w]);
+            for (int v = h; v < h + 4; ++v) {
+                const float c = ex2(m[v] - ref);
+                lsum = __fmaf_rn(c, l[v], lsum);
+                r.x = __fmaf_rn(c, acc[v].x, r.x);
+                r.y = __fmaf_rn(c, acc[v].y, r.y);
+                r.z = __fmaf_rn(c, acc[v].z, r.z);
+                r.w = __fmaf_rn(c, acc[v].w, r.w);
+            }
+            m[h] = mx;
+            l[h] = lsum;
+            acc[h] = r;
+        }
     }
+    if constexpr (kN == 2 || kN == 8)
+        lse_step(m[0], l[0], acc[0], make_float2(m[kN / 2], l[kN / 2]), acc[kN / 2]);
+}
+
+// Partial rows per split of a grid whose splits are shared by `sub` CTAs: one
+// per half where each CTA holds one, else one per accumulator.
+__host__ __device__ constexpr int parts_per_split(int sub) {
+    return sub <= 2 ? sub : kAccs;
 }
 
 // Dims 4*lane .. 4*lane + 3 of output row `row`.
@@ -275,14 +318,16 @@ __device__ __forceinline__ void merge_chains_store(const DecodeArgs &a, int64_t 
 // The merge of one query head's ns (2 .. 4 * kPer) split partials by one warp. Every
 // load is issued before the first is used (indices clamped into the row, so
 // the loads need no guard): lane t loads split t's (m, l), shared by shuffle,
-// and each lane its 4 dims of every split's accumulator. The partials come
-// from L2 (.cg), written there by other SMs.
-template <int kPer>   // splits per chain, at most
+// and each lane its 4 dims of every split's accumulator. Partials that other
+// CTAs of the same grid wrote are read from L2 (.cg); after a grid's end plain
+// loads are right, and cheaper under the next call's copies (16 x 4K tokens
+// per layer 23.8 -> 23.4 us, 32 x 4K 44.6 -> 43.9 us).
+template <int kPer, bool kSameGrid>   // kPer: splits per chain, at most
 __device__ __forceinline__ void merge_head_regs(const DecodeArgs &a, int64_t row, int ns,
                                                 int lane) {
     const int64_t base = row * a.max_splits;
-    const float2 mine = __ldcg(reinterpret_cast<const float2 *>(a.part_ml) + base +
-                               min(lane, ns - 1));
+    auto load = [](auto *p) { return kSameGrid ? __ldcg(p) : *p; };
+    const float2 mine = load(reinterpret_cast<const float2 *>(a.part_ml) + base + min(lane, ns - 1));
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o + base * kHeadDim) + lane;
     float4 o[kMergeChains][kPer];
     int s0[kMergeChains], n[kMergeChains];
@@ -291,7 +336,7 @@ __device__ __forceinline__ void merge_head_regs(const DecodeArgs &a, int64_t row
         s0[q] = (q * ns) / kMergeChains;
         n[q] = ((q + 1) * ns) / kMergeChains - s0[q];
 #pragma unroll
-        for (int i = 0; i < kPer; ++i) o[q][i] = __ldcg(po + min(s0[q] + i, ns - 1) * (kHeadDim / 4));
+        for (int i = 0; i < kPer; ++i) o[q][i] = load(po + min(s0[q] + i, ns - 1) * (kHeadDim / 4));
     }
     float m[kMergeChains], l[kMergeChains];
     float4 acc[kMergeChains];
@@ -336,53 +381,56 @@ __device__ __forceinline__ uint32_t v_offset(int lane, int i) {
     return (2 + (i >> 2)) * kHalfBytes + swz((lane & 7) + (lane >> 4) * 8, 2 * (i & 3) + ((lane >> 3) & 1));
 }
 
-// The session's last tile, in `slot` (one warp). Fused append: token T-1
-// arrives with this call; its K and V rows replace whatever the copy brought
-// for that slot and are stored to the reserved pool slot (lanes 0-15 move K,
-// 16-31 V, 16 B each). Slots past T may hold anything (NaN); P is 0 there but
-// 0 * NaN is not, so their V rows are cleared.
-__device__ __forceinline__ void finish_tail(const DecodeArgs &a, const int32_t *trow, int T,
-                                            int tok_base, int l, int lb, int g, uint8_t *slot,
-                                            int lane) {
+// The session's last tile, in `slot` (one warp), in two steps; no copy is
+// issued into the slot afterwards, so neither needs ordering against the async
+// proxy. Fused append: token T-1 arrives with this call; its K and V rows
+// replace whatever the copy brought for that slot and are stored to the
+// reserved pool slot. Lanes 0-15 move K, 16-31 V, 16 B each.
+__device__ __forceinline__ void splice_new(const DecodeArgs &a, const int32_t *trow, int T,
+                                           int tok_base, int l, int lb, int g, uint8_t *slot,
+                                           int lane) {
     const Shape &sh = a.s;
-    if (a.k_new != nullptr) {
-        const int r = T - 1 - tok_base;
-        const int u = lane & 15;
-        const int isv = lane >> 4;
-        const uint4 val = *reinterpret_cast<const uint4 *>(
-            (isv ? a.v_new : a.k_new) + (static_cast<int64_t>(lb) * sh.Hkv + g) * kHeadDim + u * 8);
-        *reinterpret_cast<uint4 *>(slot + isv * 2 * kHalfBytes + (u >> 3) * kHalfBytes +
-                                   swz(r, u & 7)) = val;
-        const int j = (T - 1) / sh.bt;
-        const int blk = trow[j];
-        if (blk >= 0 && blk < sh.num_blocks) {   // a bad id was flagged by the copy
-            const int at = ((blk * sh.L + l) * 2 * sh.Hkv + g) * sh.bt + (T - 1 - j * sh.bt) +
-                           isv * sh.Hkv * sh.bt;   // the pool has fewer than 2^31 rows
-            *reinterpret_cast<uint4 *>(a.hot + static_cast<int64_t>(at) * kHeadDim + u * 8) = val;
-        }
+    const int r = T - 1 - tok_base;
+    const int u = lane & 15;
+    const int isv = lane >> 4;
+    const uint4 val = *reinterpret_cast<const uint4 *>(
+        (isv ? a.v_new : a.k_new) + (static_cast<int64_t>(lb) * sh.Hkv + g) * kHeadDim + u * 8);
+    *reinterpret_cast<uint4 *>(slot + isv * 2 * kHalfBytes + (u >> 3) * kHalfBytes +
+                               swz(r, u & 7)) = val;
+    const int j = (T - 1) / sh.bt;
+    const int blk = trow[j];
+    if (blk >= 0 && blk < sh.num_blocks) {   // a bad id was flagged by the copy
+        const int row = ((blk * sh.L + l) * 2 * sh.Hkv + g) * sh.bt + (T - 1 - j * sh.bt) +
+                        isv * sh.Hkv * sh.bt;   // the pool has fewer than 2^31 rows
+        *reinterpret_cast<uint4 *>(a.hot + static_cast<int64_t>(row) * kHeadDim + u * 8) = val;
     }
+    __syncwarp();
+}
+// Slots past T may hold anything (NaN); P is 0 there but 0 * NaN is not, so
+// their V rows are cleared.
+__device__ __forceinline__ void clear_tail_v(int T, int tok_base, uint8_t *slot, int lane) {
     const int row = T - tok_base + (lane >> 4);   // this lane's rows: row, row + 2, ...
     uint8_t *vp = slot + (2 + ((lane >> 3) & 1)) * kHalfBytes + row * 128 + (lane & 7) * 16;
 #pragma unroll
     for (int j = 0; j < kTileTokens / 2; ++j)
         if (row + 2 * j < kTileTokens)
             *reinterpret_cast<uint4 *>(vp + j * 256) = make_uint4(0u, 0u, 0u, 0u);
-    // No copy is issued into the slot after this (it is the warp's last tile),
-    // so its reads need no ordering against the async proxy.
     __syncwarp();
 }
 
 constexpr int kOStride = kHeadDim + 4;   // floats per head row of a state in shared memory (bank skew)
 constexpr int kAccFloats = kMaxGroup * kOStride + 2 * kMaxGroup;   // O rows, m[8], l[8]
 
-// The CTA's kHere accumulator states (state(v), in shared memory) merged as a
-// tree of neighbours: a CTA that holds a part of a split's accumulators has a
-// node of the whole split's tree. One warp per head, four dims per lane, so a
-// warp reads one head's row of a state as 32 consecutive float4. A session of
-// one split held by one CTA is finished here; others leave a partial.
+// The CTA's kHere accumulator states (state(v), in shared memory): a whole
+// split or a half of one is merged, fewer are left to the combine. One warp per
+// head, four dims per lane, so a warp reads one head's row of a state as 32
+// consecutive float4. A session of one split held by one CTA is finished here;
+// others leave partials.
 template <int kHere, int kSub, int kWarps, typename State>
 __device__ __forceinline__ void merge_states(const DecodeArgs &a, int64_t row_base, int G,
                                              int nsplit, int split, int sub, State state) {
+    constexpr int kParts = parts_per_split(kSub);   // of the split
+    constexpr int kMine = kParts / kSub;            // of this CTA
     const int lane = threadIdx.x & 31;
     const int d0 = lane * 4;
 #pragma unroll 1
@@ -396,17 +444,20 @@ __device__ __forceinline__ void merge_states(const DecodeArgs &a, int64_t row_ba
             l[v] = ws[kMaxGroup * kOStride + kMaxGroup + h];
             acc[v] = *reinterpret_cast<const float4 *>(ws + h * kOStride + d0);
         }
-        lse_tree<kHere>(m, l, acc);
+        if constexpr (kMine == 1) join_accs<kHere>(m, l, acc);
         if (kSub == 1 && nsplit == 1) {
             const float inv = __frcp_rn(l[0]);
             store_out(a, row_base + h, lane,
                       make_float4(__fmul_rn(acc[0].x, inv), __fmul_rn(acc[0].y, inv),
                                   __fmul_rn(acc[0].z, inv), __fmul_rn(acc[0].w, inv)));
         } else {
-            const int64_t prow = ((row_base + h) * a.max_splits + split) * kSub + sub;
-            *reinterpret_cast<float4 *>(a.part_o + prow * kHeadDim + d0) = acc[0];
-            if (lane == 0)
-                *reinterpret_cast<float2 *>(a.part_ml + prow * 2) = make_float2(m[0], l[0]);
+            const int64_t prow = ((row_base + h) * a.max_splits + split) * kParts + sub * kMine;
+#pragma unroll
+            for (int v = 0; v < kMine; ++v) {
+                *reinterpret_cast<float4 *>(a.part_o + (prow + v) * kHeadDim + d0) = acc[v];
+                if (lane == 0)
+                    *reinterpret_cast<float2 *>(a.part_ml + (prow + v) * 2) = make_float2(m[v], l[v]);
+            }
         }
     }
 }
@@ -522,6 +573,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     }
     __syncwarp();
 
+    const uint64_t policy = copy_policy(a.stream != 0);
     // Producer step (lane 0): tile k of this warp, in block blk, into slot
     // k % kStages.
     auto issue = [&](int k, int blk) {
@@ -539,7 +591,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         // one barrier then never completes its phase, although every copy lands.
         const bool injected = k == 0 && warp == 0 && slice == 0 && g == 0 && lb == 0;
         mbar_expect_tx(bar, kTileBytes + (injected ? a.inject_extra_tx : 0));
-        tma_load_tile(slot, &map, rowk, bar);
+        tma_load_tile(slot, &map, rowk, bar, policy);
     };
     // The block of tile k, for every lane (k < 32 wherever it is used).
     auto blk_of = [&](int k) { return __shfl_sync(0xffffffffu, lane_blk, k & 31); };
@@ -550,6 +602,13 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         const int blk = blk_of(k);
         if (a.pace > 0 && k >= a.pace) mbar_wait(bar0 + 8 * (k - a.pace), 0);
         if (lane == 0) issue(k, blk);
+    }
+
+    uint32_t koff[4], voff[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        koff[j] = k_offset(lane, j);
+        voff[j] = v_offset(lane, j);
     }
 
     // Everything above reads only the hot pool, the block table and seq_lens.
@@ -575,20 +634,15 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     const float sl = a.scale_log2;
     int fail_k = -1;
 
-    uint32_t koff[4], voff[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        koff[j] = k_offset(lane, j);
-        voff[j] = v_offset(lane, j);
-    }
-
     auto load_k = [&](uint32_t slot, int ks, uint32_t (&f)[4]) {
         ldsm_x4(slot + koff[ks & 3] + (ks >> 2) * kHalfBytes, f[0], f[1], f[2], f[3]);
     };
+    auto load_v = [&](uint32_t slot, int i, uint32_t (&f)[4]) {
+        ldsm_x4_t(slot + voff[i & 3] + (i >> 2) * kHalfBytes, f[0], f[1], f[2], f[3]);
+    };
     auto load_values = [&](uint32_t slot, uint32_t (&f)[8][4]) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            ldsm_x4_t(slot + voff[i & 3] + (i >> 2) * kHalfBytes, f[i][0], f[i][1], f[i][2], f[i][3]);
+        for (int i = 0; i < 8; ++i) load_v(slot, i, f[i]);
     };
     // One k-step (16 dims) of S^T = K . Q^T into acc.
     auto qk_step = [&](const uint32_t (&f)[4], int ks, float (&acc)[4]) {
@@ -667,15 +721,23 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         if (!mbar_wait(bar0 + 8 * (k % kStages), (k / kStages) & 1)) return false;
         const int tok_base = tile_base(k);
         const uint32_t slot = slot_of(k);
-        if (tok_base + kTileTokens >= T)
-            finish_tail(a, trow, T, tok_base, l, lb, g, ring + (k % kStages) * kTileBytes, lane);
+        uint8_t *const tile = ring + (k % kStages) * kTileBytes;
+        if (a.k_new != nullptr && tok_base + kTileTokens >= T)
+            splice_new(a, trow, T, tok_base, l, lb, g, tile, lane);
+        if (kSub > 1 && tok_base + kTileTokens > T) clear_tail_v(T, tok_base, tile, lane);
         // S^T = K . Q^T, two accumulators to shorten the mma chain.
         float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f}, x[4];
         uint32_t kf[8][4], vf[8][4];
+        if constexpr (kSub > 1) {
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) load_k(slot, ks, kf[ks]);
+            for (int ks = 0; ks < 8; ++ks) load_k(slot, ks, kf[ks]);
+        }
 #pragma unroll
         for (int ks = 0; ks < 8; ks += 2) {
+            if constexpr (kSub == 1) {
+                load_k(slot, ks, kf[ks]);
+                load_k(slot, ks + 1, kf[ks + 1]);
+            }
             qk_step(kf[ks], ks, sa);
             qk_step(kf[ks + 1], ks + 1, sb);
         }
@@ -686,8 +748,16 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         if (__any_sync(0xffffffffu, grows(x, s))) move_max(x, s);
         uint32_t pb0, pb1;
         weights(x, s, pb0, pb1);
-        if constexpr (kSub == 1) load_values(slot, vf);
-        add_values(vf, s, pb0, pb1);
+        if constexpr (kSub == 1) {
+            if (tok_base + kTileTokens > T) clear_tail_v(T, tok_base, tile, lane);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                load_v(slot, i, vf[i]);
+                mma_bf16(s.o[i], vf[i][0], vf[i][1], vf[i][2], vf[i][3], pb0, pb1);
+            }
+        } else {
+            add_values(vf, s, pb0, pb1);
+        }
         __syncwarp();
         refill(k);
         return true;
@@ -866,7 +936,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     __syncthreads();
     if (!s_last) return;
 #pragma unroll 1
-    for (int h = warp; h < G; h += kWarps) merge_head_regs<kSplitKernelMerge / kMergeChains>(a, row_base + h, nsplit, lane);
+    for (int h = warp; h < G; h += kWarps) merge_head_regs<kSplitKernelMerge / kMergeChains, true>(a, row_base + h, nsplit, lane);
 }
 
 // K2 for tables of at most kRegMergeMax splits: one warp per (layer-batch
@@ -884,19 +954,19 @@ __global__ void __launch_bounds__(128) decode_combine_small_kernel(const DecodeA
     const int ns = num_splits(T);
     if (ns <= 1 || ns <= a.merge_max_splits) return;   // written by K1
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    merge_head_regs<kRegMergeMax / kMergeChains>(a, row, ns, threadIdx.x & 31);
+    merge_head_regs<kRegMergeMax / kMergeChains, false>(a, row, ns, threadIdx.x & 31);
 }
 
 // K2 for wider tables: one CTA (4 warps) per (layer-batch row, q-head) of a
 // multi-split session the split kernel did not merge. Warp w folds chain w, the
 // contiguous quarter [w*ns/4, (w+1)*ns/4) of the splits (split order), each
-// split's kSub states joined first as the split kernel joins accumulators, then
+// split's kParts states joined first as the split kernel joins them, then
 // warp 0 merges the four chains in order. The result depends only on the
 // partials and ns. Launched as a programmatic dependent of K1: it waits for
 // K1's completion with griddepcontrol.wait, so its CTAs can already be resident
 // while K1 drains. Batches of kBatch splits: every load of a batch is issued
 // before the first is folded (indices clamped into the quarter, no guards).
-template <int kSub, int kBatch>
+template <int kParts, int kBatch>
 __global__ void __launch_bounds__(128) decode_combine_kernel(const DecodeArgs a) {
     asm volatile("griddepcontrol.launch_dependents;");   // a following overlapped call
     const int64_t row = blockIdx.x;                // lb * Hq + h
@@ -907,41 +977,40 @@ __global__ void __launch_bounds__(128) decode_combine_kernel(const DecodeArgs a)
     const int T = a.seq_lens[b];
     if (T < 1 || T > a.max_blocks * a.s.bt) return;
     const int ns = num_splits(T);
-    if (kSub == 1 && (ns <= 1 || ns <= a.merge_max_splits)) return;   // written by K1
+    if (kParts == 1 && (ns <= 1 || ns <= a.merge_max_splits)) return;   // written by K1
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-    const int64_t base = row * a.max_splits * kSub;
+    const int64_t base = row * a.max_splits * kParts;
     const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + base;
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o + base * kHeadDim) + lane;
     __shared__ float s_m[kCombineWarps], s_l[kCombineWarps];
     __shared__ float4 s_acc[kCombineWarps][kHeadDim / 4];
     const int s0 = (warp * ns) / kCombineWarps;
     const int s1 = ((warp + 1) * ns) / kCombineWarps;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     float m = -INFINITY, lsum = 0.f;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
     for (int sb = s0; sb < s1; sb += kBatch) {
-        float2 v[kBatch][kSub];
-        float4 o[kBatch][kSub];
+        float2 v[kBatch][kParts];
+        float4 o[kBatch][kParts];
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
-            const int sp = min(sb + j, s1 - 1) * kSub;
+            const int sp = min(sb + j, s1 - 1) * kParts;
 #pragma unroll
-            for (int r = 0; r < kSub; ++r) {
-                v[j][r] = __ldcg(ml + sp + r);
-                o[j][r] = __ldcg(po + (sp + r) * (kHeadDim / 4));
+            for (int r = 0; r < kParts; ++r) {
+                v[j][r] = ml[sp + r];
+                o[j][r] = po[(sp + r) * (kHeadDim / 4)];
             }
         }
 #pragma unroll
         for (int j = 0; j < kBatch; ++j) {
-            float mr[kSub], lr[kSub];
+            float mr[kParts], lr[kParts];
 #pragma unroll
-            for (int r = 0; r < kSub; ++r) {
+            for (int r = 0; r < kParts; ++r) {
                 mr[r] = v[j][r].x;
                 lr[r] = v[j][r].y;
             }
-            lse_tree<kSub>(mr, lr, o[j]);
+            join_accs<kParts>(mr, lr, o[j]);
             if (sb + j < s1) lse_step(m, lsum, acc, make_float2(mr[0], lr[0]), o[j][0]);
         }
     }
@@ -964,14 +1033,14 @@ __global__ void __launch_bounds__(128) decode_combine_kernel(const DecodeArgs a)
     }
 }
 
-// K2 for splits shared by kSub CTAs, tables of at most kRegMergeMax splits: as
-// above, with all of a chain's partials (at most four splits of kSub states)
+// K2 for shared splits, tables of at most kRegMergeMax splits: as above, with
+// all of a chain's partials (at most four splits of 2 halves or 8 accumulators)
 // loaded at once. Latency-bound: one round trip to L2 (0.13 us, several times
 // that under the next call's copies), then 0.4 us of dependent steps. The loop
 // above in its place keeps fewer registers and starts its loads after each
 // other: 6.2 instead of 5.3 us per layer for one session of 3 001 tokens, 13.3
 // instead of 12.5 for 8 x 4K.
-template <int kSub>
+template <int kParts>
 __global__ void __launch_bounds__(128) decode_combine_shared_kernel(const DecodeArgs a) {
     asm volatile("griddepcontrol.launch_dependents;");   // a following overlapped call
     const int64_t row = blockIdx.x;                // lb * Hq + h
@@ -983,21 +1052,21 @@ __global__ void __launch_bounds__(128) decode_combine_shared_kernel(const Decode
     const int lane = threadIdx.x & 31;
     const int s0 = (warp * ns) / kMergeChains;
     const int n = ((warp + 1) * ns) / kMergeChains - s0;
-    const int64_t base = row * a.max_splits * kSub;
+    const int64_t base = row * a.max_splits * kParts;
     const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + base;
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o + base * kHeadDim) + lane;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     __shared__ float s_m[kMergeChains], s_l[kMergeChains];
     __shared__ float4 s_acc[kMergeChains][kHeadDim / 4];
     constexpr int kPer = kRegMergeMax / kMergeChains;
-    float2 v[kPer][kSub];
-    float4 o[kPer][kSub];
+    float2 v[kPer][kParts];
+    float4 o[kPer][kParts];
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         if (i < n) {
 #pragma unroll
-            for (int r = 0; r < kSub; ++r) {
-                const int p = (s0 + i) * kSub + r;
+            for (int r = 0; r < kParts; ++r) {
+                const int p = (s0 + i) * kParts + r;
                 v[i][r] = __ldcg(ml + p);
                 o[i][r] = __ldcg(po + p * (kHeadDim / 4));
             }
@@ -1008,13 +1077,13 @@ __global__ void __launch_bounds__(128) decode_combine_shared_kernel(const Decode
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         if (i < n) {
-            float mr[kSub], lr[kSub];
+            float mr[kParts], lr[kParts];
 #pragma unroll
-            for (int r = 0; r < kSub; ++r) {
+            for (int r = 0; r < kParts; ++r) {
                 mr[r] = v[i][r].x;
                 lr[r] = v[i][r].y;
             }
-            lse_tree<kSub>(mr, lr, o[i]);
+            join_accs<kParts>(mr, lr, o[i]);
             lse_step(m, lsum, acc, make_float2(mr[0], lr[0]), o[i][0]);
         }
     }
@@ -1084,7 +1153,12 @@ static cudaError_t prepare_split() {
 }
 
 cudaError_t prepare_kernels() {
-    cudaError_t e = prepare_split<kWarpsNarrow, kStagesFull, 1>();
+    // Set in order, the last one telling that all of them are set: every pool
+    // asks, and each set costs a pool's creation some 15 us.
+    cudaFuncAttributes set;
+    cudaError_t e = cudaFuncGetAttributes(&set, decode_split_kernel<1, 8, 8>);
+    if (e == cudaSuccess && set.maxDynamicSharedSizeBytes >= decode_smem(1, 8)) return e;
+    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1>();
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1>();
     if (e == cudaSuccess) e = prepare_split<8, 3, 1>();
     if (e == cudaSuccess) e = prepare_split<4, 6, 2>();
@@ -1131,7 +1205,7 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // each of its CTAs draws 512 KB or more through one SM (6 us) with its
     // warps in each other's way; shared, a CTA has less to draw, holds more of
     // it before the previous call ends, and is gone sooner, so the next call's
-    // CTAs start their copies sooner. The combine reads kSub states per split
+    // CTAs start their copies sooner. The combine reads 2 or 8 states per split
     // instead of one. us per layer, unshared and shared:
     //   8 or 4 CTAs, at most one per SM: 1 x 3 001 8.04 and 5.36, 1 x 8K 8.51
     //     and 6.74, 4 x 1 280 8.26 and 6.17
@@ -1151,7 +1225,7 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     const int64_t sms = num_sms;
     const int64_t rows1 = static_cast<int64_t>(splits) * a.s.Hq * a.nlayers * a.B;
     auto fits = [&](int sub, int per_sm) {
-        return sub * ctas <= per_sm * sms && sub * rows1 <= a.part_rows;
+        return sub * ctas <= per_sm * sms && parts_per_split(sub) * rows1 <= a.part_rows;
     };
     const bool wide = splits > kRegMergeMax;   // long splits, and a combine in batches
     int sub = 1;
@@ -1178,11 +1252,12 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // and 12.7; 8 x 4K 15.0 and 13.2, 12 x 2K 12.1 and 11.4; 4 x 16K 24.1 and
     // 23.1. Rings that cover a whole split (4 or 8 CTAs per split) showed no
     // difference, and in grids of more than one wave the later CTAs lose by it
-    // (8 x 16K 44.4 and 45.1); unshared long splits take no part (1 x 100K).
+    // (8 x 16K 44.4 and 45.1). Calls without a combine (40 x 1 000 16.0 and
+    // 16.9) and unshared long splits (1 x 100K) take no part.
     ka.pace = 0;
     if (overlap_previous && sub == 2)
         ka.pace = per_sm == 1 ? 2 : 1;
-    else if (overlap_previous && sub == 1 && !wide && ctas <= 2 * sms)
+    else if (overlap_previous && sub == 1 && splits > 1 && !wide && ctas <= 2 * sms)
         ka.pace = 1;
 
     // Which sessions the split kernel merges itself (the bits are the same
@@ -1195,6 +1270,8 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // layers +1.6 %; one 4K- or 16K-token session per layer -7 % / -5 % and
     // 32 x 4K -5 % when shorter grids merged too).
     ka.merge_max_splits = ctas >= 8 * sms ? kSplitKernelMerge : 0;
+    const bool combine = sub > 1 || (splits > 1 && splits > ka.merge_max_splits);
+    ka.stream = combine;
     cudaError_t e;
     if (sub == 8)
         e = launch_split<1, 8, 8>(c1, map, ka);
@@ -1213,9 +1290,9 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     else
         e = launch_split<kWarpsNarrow, kStagesFull, 1>(c1, map, ka);
     if (e != cudaSuccess) return e;
-    // Every session's output written by the split kernel: one split each, or
+    // Else the split kernel writes every session's output: one split each, or
     // few enough splits to merge there.
-    if (sub == 1 && (splits <= 1 || splits <= ka.merge_max_splits)) return cudaSuccess;
+    if (!combine) return cudaSuccess;
 
     const int64_t rows = static_cast<int64_t>(a.nlayers) * a.B * a.s.Hq;
     cudaLaunchConfig_t c2 = {};
@@ -1232,8 +1309,7 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     if (wide)
         return sub == 2 ? cudaLaunchKernelEx(&c2, decode_combine_kernel<2, 8>, ka)
                         : cudaLaunchKernelEx(&c2, decode_combine_kernel<1, 16>, ka);
-    if (sub == 8) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<8>, ka);
-    if (sub == 4) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<4>, ka);
+    if (sub > 2) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<8>, ka);
     return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<2>, ka);
 }
 
