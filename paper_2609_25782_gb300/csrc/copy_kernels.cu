@@ -8,6 +8,7 @@
 //   block_jobs_kernel<>    the same moves for explicit (slot, block, token
 //                          range) lists: residency-mode evictions and fetches.
 //   append_kernel          data path 3: fresh tokens into the tail blocks.
+//   append_inline_kernel   the same with up to 2 048 new block ids in the launch.
 //   table_write_kernel / gather_tables_kernel: block-table bookkeeping.
 //
 // Hot pool: hot[NB][L][2][Hkv][bt][128] bf16. A (block, layer, K|V, head)
@@ -19,26 +20,49 @@
 namespace kvt {
 namespace {
 
-// Migration copy shape, from GB300 measurements of 2..16 loads per lane and
-// 4..32 CTAs per SM: 4 loads per lane over a grid of 32 CTAs per SM, one warp
-// per 16-token chunk of a run, moves an 8 x 32K-token burst at the copy
-// bandwidth (0.93 of it with 8 loads x 8 CTAs).
+// Migration copy shape: one warp per 16-token chunk of a run (4 KiB on both
+// sides), moved by one round of 32-byte loads, four per lane, and stores. Bound
+// by HBM. The warps are not reused: a grid-stride loop over 32 CTAs per SM moved
+// three sessions of 20K-30K tokens in 2.26 ms, one warp per chunk in 2.19 ms
+// (its 16-byte predecessor in 2.31 ms, 1.00 of the copy bandwidth).
+// Moves larger than kOnceBytes touch image and blocks once and let both leave
+// the L2 first, which leaves room for what others keep there: of a turn of
+// 1 536 tokens, appended and then packed, the pack finds most of the appended
+// blocks in the L2 (96.1 -> 87.4 us with both hints, 94.4 with one of them).
+// Smaller ones may be used again while they are there (two resumes of 300
+// tokens 26.4 us, 28.0 with the hints).
 constexpr int kMigChunkTokens = 16;     // tokens per migration item (divides bt)
-#ifndef KVT_MIG_UNROLL
-#define KVT_MIG_UNROLL 4          // 16-byte loads in flight per lane
-#endif
-#ifndef KVT_MIG_CTAS_PER_SM
-#define KVT_MIG_CTAS_PER_SM 32    // grid-stride CTAs of 256 threads per SM
-#endif
+constexpr int kMigUnroll = 4;           // 32-byte loads in flight per lane
+static_assert(kMigChunkTokens * kRowBytes == 32 * 32 * kMigUnroll, "one round moves a chunk");
+constexpr int64_t kOnceBytes = int64_t(32) << 20;   // a quarter of the L2
+constexpr int kAppendUnroll = 4;        // 16-byte loads in flight per lane
 
-__device__ __forceinline__ void st_out(uint4 *p, const uint4 &v) {
-#ifdef KVT_MIG_STREAM_STORE
-    asm volatile("st.global.cs.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y),
-                 "r"(v.z), "r"(v.w)
+struct alignas(32) Row32 {
+    uint32_t w[8];
+};
+
+// L2 policies of a move: its lines leave first, or as any others.
+__device__ __forceinline__ uint64_t move_policy(bool once) {
+    uint64_t p, q;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(q));
+    return once ? p : q;
+}
+
+__device__ __forceinline__ Row32 ld_row(const Row32 *p, uint64_t policy) {
+    Row32 v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], %9;"
+                 : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]),
+                   "=r"(v.w[5]), "=r"(v.w[6]), "=r"(v.w[7])
+                 : "l"(p), "l"(policy));
+    return v;
+}
+
+__device__ __forceinline__ void st_row(Row32 *p, const Row32 &v, uint64_t policy) {
+    asm volatile("st.global.L2::cache_hint.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8}, %9;" ::"l"(p),
+                 "r"(v.w[0]), "r"(v.w[1]), "r"(v.w[2]), "r"(v.w[3]), "r"(v.w[4]), "r"(v.w[5]),
+                 "r"(v.w[6]), "r"(v.w[7]), "l"(policy)
                  : "memory");
-#else
-    *p = v;
-#endif
 }
 
 __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
@@ -49,10 +73,26 @@ __device__ __forceinline__ uint4 ld_stream(const uint4 *p) {
     return v;
 }
 
-// K3 / K4: one warp per (layer, K|V, kv-head, block) run of the token range.
-// Both sides of a run are contiguous rows of 256 B; a warp moves it with
-// 16-byte loads, KVT_MIG_UNROLL in flight per lane. Items are ordered run-major so
-// that consecutive warps walk the image sequentially.
+// Up to one chunk of rows from `from` to `to` by a warp.
+__device__ __forceinline__ void move_rows(const uint8_t *from, uint8_t *to, int rows, int lane,
+                                          uint64_t policy) {
+    const Row32 *src = reinterpret_cast<const Row32 *>(from) + lane;
+    Row32 *dst = reinterpret_cast<Row32 *>(to) + lane;
+    const int units = rows * (kRowBytes / 32) - lane;
+    Row32 v[kMigUnroll];
+#pragma unroll
+    for (int k = 0; k < kMigUnroll; ++k)
+        if (k * 32 < units) v[k] = ld_row(src + k * 32, policy);
+#pragma unroll
+    for (int k = 0; k < kMigUnroll; ++k)
+        if (k * 32 < units) st_row(dst + k * 32, v[k], policy);
+}
+
+// K3 / K4: the chunks of the token range of every (layer, K|V, kv-head) run.
+// Both sides of a chunk are contiguous rows of 256 B. Items are ordered
+// run-major so that consecutive warps walk the image sequentially (the eight
+// runs of a block next to each other instead: 4.39 against 4.37 ms for the
+// sessions above).
 // The copy loop of a session's migration; block_of(j) gives logical block j's slot.
 template <bool kPack, typename BlockOf>
 __device__ __forceinline__ void migrate_runs(const MigArgs &a, BlockOf block_of) {
@@ -65,6 +105,7 @@ __device__ __forceinline__ void migrate_runs(const MigArgs &a, BlockOf block_of)
     const int nq = q1 - q0;
     const int items = runs * nq;
     const int lane = threadIdx.x & 31;
+    const uint64_t policy = move_policy(a.once);
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += nwarps) {
         const int c = it / nq;
@@ -80,22 +121,7 @@ __device__ __forceinline__ void migrate_runs(const MigArgs &a, BlockOf block_of)
         uint8_t *hp = a.hot + ((static_cast<int64_t>(blk) * runs + c) * sh.bt + (t_lo - j * sh.bt)) *
                                   kRowBytes;
         uint8_t *ip = a.img + (static_cast<int64_t>(c) * a.T_cap + t_lo) * kRowBytes;
-        const uint4 *src = reinterpret_cast<const uint4 *>(kPack ? hp : ip);
-        uint4 *dst = reinterpret_cast<uint4 *>(kPack ? ip : hp);
-        const int units = (t_hi - t_lo) * (kRowBytes / 16);
-        for (int u0 = 0; u0 < units; u0 += 32 * KVT_MIG_UNROLL) {
-            uint4 v[KVT_MIG_UNROLL];
-#pragma unroll
-            for (int k = 0; k < KVT_MIG_UNROLL; ++k) {
-                const int u = u0 + k * 32 + lane;
-                if (u < units) v[k] = ld_stream(src + u);
-            }
-#pragma unroll
-            for (int k = 0; k < KVT_MIG_UNROLL; ++k) {
-                const int u = u0 + k * 32 + lane;
-                if (u < units) st_out(dst + u, v[k]);
-            }
-        }
+        move_rows(kPack ? hp : ip, kPack ? ip : hp, t_hi - t_lo, lane, policy);
     }
 }
 
@@ -123,6 +149,7 @@ __global__ void __launch_bounds__(256) block_jobs_kernel(const __grid_constant__
     const int cpb = sh.bt / kMigChunkTokens;      // 16-token chunks per block
     const int items = a.n * runs * cpb;
     const int lane = threadIdx.x & 31;
+    const uint64_t policy = move_policy(a.once);
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += nwarps) {
         const int jb = it / (runs * cpb);
@@ -142,22 +169,7 @@ __global__ void __launch_bounds__(256) block_jobs_kernel(const __grid_constant__
         uint8_t *hp = a.hot + ((static_cast<int64_t>(b.slot) * runs + c) * sh.bt + t_lo) * kRowBytes;
         uint8_t *ip = b.img + (static_cast<int64_t>(c) * b.T_cap + static_cast<int64_t>(b.j) * sh.bt +
                                t_lo) * kRowBytes;
-        const uint4 *src = reinterpret_cast<const uint4 *>(kPack ? hp : ip);
-        uint4 *dst = reinterpret_cast<uint4 *>(kPack ? ip : hp);
-        const int units = (t_hi - t_lo) * (kRowBytes / 16);
-        for (int u0 = 0; u0 < units; u0 += 32 * KVT_MIG_UNROLL) {
-            uint4 v[KVT_MIG_UNROLL];
-#pragma unroll
-            for (int k = 0; k < KVT_MIG_UNROLL; ++k) {
-                const int u = u0 + k * 32 + lane;
-                if (u < units) v[k] = ld_stream(src + u);
-            }
-#pragma unroll
-            for (int k = 0; k < KVT_MIG_UNROLL; ++k) {
-                const int u = u0 + k * 32 + lane;
-                if (u < units) st_out(dst + u, v[k]);
-            }
-        }
+        move_rows(kPack ? hp : ip, kPack ? ip : hp, t_hi - t_lo, lane, policy);
     }
 }
 
@@ -167,7 +179,9 @@ __global__ void __launch_bounds__(256) block_jobs_kernel(const __grid_constant__
 // One warp per (layer, token) item, items layer-major so that consecutive
 // warps read k and v sequentially. A lane issues all of its 16-byte loads of
 // the item (K and V rows of every kv-head) before its first store.
-__global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
+// block_of(j) gives logical block j's slot.
+template <typename BlockOf>
+__device__ __forceinline__ void append_tokens(const AppendArgs &a, BlockOf block_of) {
     const Shape sh = a.s;
     const int items = sh.L * a.n;
     const int lane = threadIdx.x & 31;
@@ -180,7 +194,7 @@ __global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
         const int64_t src_off = static_cast<int64_t>(it) * sh.Hkv * kRowBytes;
         const uint4 *ks = reinterpret_cast<const uint4 *>(a.k + src_off);
         const uint4 *vs = reinterpret_cast<const uint4 *>(a.v + src_off);
-        const int blk = a.table[t / sh.bt];
+        const int blk = block_of(static_cast<int>(t / sh.bt));
         const bool ok = blk >= 0 && blk < sh.num_blocks;
         if (!ok && lane == 0) atomicOr(a.err, kErrBadBlock);
         // Unit u = (kv * Hkv + g) * 16 + c lands in run (kv, g), row `slot`.
@@ -188,22 +202,40 @@ __global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
         uint8_t *base = a.hot + ((static_cast<int64_t>(ok ? blk : 0) * sh.L + l) * 2 * sh.Hkv *
                                      sh.bt + slot) * kRowBytes;
         const int64_t run_bytes = static_cast<int64_t>(sh.bt) * kRowBytes;
-        for (int u0 = 0; u0 < 2 * units; u0 += 32 * KVT_MIG_UNROLL) {
-            uint4 v[KVT_MIG_UNROLL];
+        for (int u0 = 0; u0 < 2 * units; u0 += 32 * kAppendUnroll) {
+            uint4 v[kAppendUnroll];
 #pragma unroll
-            for (int k = 0; k < KVT_MIG_UNROLL; ++k) {
+            for (int k = 0; k < kAppendUnroll; ++k) {
                 const int u = u0 + k * 32 + lane;
                 if (u < 2 * units) v[k] = ld_stream(u < units ? ks + u : vs + (u - units));
             }
             if (!ok) continue;
 #pragma unroll
-            for (int k = 0; k < KVT_MIG_UNROLL; ++k) {
+            for (int k = 0; k < kAppendUnroll; ++k) {
                 const int u = u0 + k * 32 + lane;
                 if (u < 2 * units)
-                    st_out(reinterpret_cast<uint4 *>(base + (u >> 4) * run_bytes) + (u & 15), v[k]);
+                    reinterpret_cast<uint4 *>(base + (u >> 4) * run_bytes)[u & 15] = v[k];
             }
         }
     }
+}
+
+__global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
+    append_tokens(a, [&](int j) { return a.table[j]; });
+}
+
+// An append whose new block ids ride in the launch: the grid also writes them
+// to the session's table row (read by later work only), which saves the
+// table-write launch in front of it: a turn of 1 536 tokens, appended and
+// packed, 98.5 -> KVT_TURN us.
+__global__ void __launch_bounds__(256) append_inline_kernel(const __grid_constant__ AppendInlineArgs r) {
+    const int nthreads = gridDim.x * blockDim.x;
+    int32_t *row = const_cast<int32_t *>(r.m.table);   // the pool's own row: writable
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < r.n; j += nthreads)
+        row[r.from + j] = r.blocks[j];
+    append_tokens(r.m, [&](int j) {
+        return j < r.from ? r.m.table[j] : j < r.from + r.n ? r.blocks[j - r.from] : -1;
+    });
 }
 
 __global__ void table_write_kernel(const __grid_constant__ TableWriteArgs a) {
@@ -227,52 +259,63 @@ __global__ void gather_tables_kernel(const __grid_constant__ GatherArgs a) {
 
 }  // namespace
 
-// One warp per item, 8 per CTA; at most KVT_MIG_CTAS_PER_SM per SM, or
-// max_ctas when the caller caps migrations (max_ctas > 0).
-static unsigned mig_grid(int64_t items, int num_sms, int max_ctas) {
+// One warp per item, 8 per CTA; at most `cap` CTAs (0: as many as a thread
+// index of 31 bits counts). The kernels stride over what is left.
+constexpr int64_t kMaxCtas = int64_t(1) << 23;
+static unsigned item_grid(int64_t items, int64_t cap) {
     int64_t blocks = (items + 7) / 8;
-    int64_t cap = static_cast<int64_t>(num_sms) * KVT_MIG_CTAS_PER_SM;
-    if (max_ctas > 0 && max_ctas < cap) cap = max_ctas;
+    if (cap <= 0 || cap > kMaxCtas) cap = kMaxCtas;
     if (blocks > cap) blocks = cap;
     return static_cast<unsigned>(blocks < 1 ? 1 : blocks);
 }
 
-cudaError_t launch_unpack(const MigArgs &a, int num_sms, int max_ctas, cudaStream_t st) {
+// Chunks of a session's move, and whether it goes through the L2 once.
+static int64_t move_items(const MigArgs &a) {
+    const int64_t nq = (a.t_end + kMigChunkTokens - 1) / kMigChunkTokens - a.t_begin / kMigChunkTokens;
+    return nq * a.s.L * 2 * a.s.Hkv;
+}
+static int32_t moves_once(int64_t items) {
+    return items * kMigChunkTokens * kRowBytes > kOnceBytes;
+}
+
+cudaError_t launch_unpack(MigArgs a, int max_ctas, cudaStream_t st) {
     if (a.t_end <= a.t_begin) return cudaSuccess;
-    const int64_t nq = (a.t_end + kMigChunkTokens - 1) / kMigChunkTokens - a.t_begin / kMigChunkTokens;
-    migrate_kernel<false><<<mig_grid(nq * a.s.L * 2 * a.s.Hkv, num_sms, max_ctas), 256, 0, st>>>(a);
+    a.once = moves_once(move_items(a));
+    migrate_kernel<false><<<item_grid(move_items(a), max_ctas), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_unpack_inline(const ResumeArgs &r, int num_sms, int max_ctas, cudaStream_t st) {
-    const MigArgs &a = r.m;
-    if (a.t_end <= a.t_begin || r.n < 1 || r.n > kResumeInlineMax) return cudaErrorInvalidValue;
-    const int64_t nq = (a.t_end + kMigChunkTokens - 1) / kMigChunkTokens - a.t_begin / kMigChunkTokens;
-    resume_inline_kernel<<<mig_grid(nq * a.s.L * 2 * a.s.Hkv, num_sms, max_ctas), 256, 0, st>>>(r);
+cudaError_t launch_unpack_inline(ResumeArgs &r, int max_ctas, cudaStream_t st) {
+    if (r.m.t_end <= r.m.t_begin || r.n < 1 || r.n > kResumeInlineMax) return cudaErrorInvalidValue;
+    r.m.once = moves_once(move_items(r.m));
+    resume_inline_kernel<<<item_grid(move_items(r.m), max_ctas), 256, 0, st>>>(r);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack(const MigArgs &a, int num_sms, int max_ctas, cudaStream_t st) {
+cudaError_t launch_pack(MigArgs a, int max_ctas, cudaStream_t st) {
     if (a.t_end <= a.t_begin) return cudaSuccess;
-    const int64_t nq = (a.t_end + kMigChunkTokens - 1) / kMigChunkTokens - a.t_begin / kMigChunkTokens;
-    migrate_kernel<true><<<mig_grid(nq * a.s.L * 2 * a.s.Hkv, num_sms, max_ctas), 256, 0, st>>>(a);
+    a.once = moves_once(move_items(a));
+    migrate_kernel<true><<<item_grid(move_items(a), max_ctas), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_append(const AppendArgs &a, int num_sms, cudaStream_t st) {
-    const int64_t warps = static_cast<int64_t>(a.s.L) * a.n;
-    int64_t blocks = (warps + 7) / 8;
-    const int64_t cap = static_cast<int64_t>(num_sms) * KVT_MIG_CTAS_PER_SM;
-    if (blocks > cap) blocks = cap;
-    append_kernel<<<static_cast<unsigned>(blocks < 1 ? 1 : blocks), 256, 0, st>>>(a);
+cudaError_t launch_append(const AppendArgs &a, cudaStream_t st) {
+    append_kernel<<<item_grid(static_cast<int64_t>(a.s.L) * a.n, 0), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_block_jobs(const BlockJobs &a, bool pack, int num_sms, int max_ctas,
-                              cudaStream_t st) {
+cudaError_t launch_append_inline(const AppendInlineArgs &r, cudaStream_t st) {
+    if (r.n < 1 || r.n > kResumeInlineMax) return cudaErrorInvalidValue;
+    append_inline_kernel<<<item_grid(static_cast<int64_t>(r.m.s.L) * r.m.n, 0), 256, 0, st>>>(r);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_block_jobs(BlockJobs &a, bool pack, int max_ctas, cudaStream_t st) {
     if (a.n <= 0) return cudaSuccess;
-    const unsigned grid = mig_grid(static_cast<int64_t>(a.n) * a.s.L * 2 * a.s.Hkv *
-                                       (a.s.bt / kMigChunkTokens), num_sms, max_ctas);
+    const int64_t items = static_cast<int64_t>(a.n) * a.s.L * 2 * a.s.Hkv *
+                          (a.s.bt / kMigChunkTokens);
+    const unsigned grid = item_grid(items, max_ctas);
+    a.once = moves_once(items);
     if (pack)
         block_jobs_kernel<true><<<grid, 256, 0, st>>>(a);
     else

@@ -135,9 +135,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 // L2 for 32 sessions of 20K tokens) also pushes out the partials, which the
 // combine then reads from HBM behind the next call's copies: us per layer with
 // the default policy and this one, 16 x 14K tokens 72.7 and 70.2, 32 x 20K 191
-// and 185.5, 64 x 8K 154.3 and 150.4, 8 x 16K 45.2 and 44.1; sessions whose
-// layer fits the L2 the same. Calls that leave no partials for a combine keep
-// the default (256 x 1 000 81.1 and 82.0).
+// and 185.5, 64 x 8K 154.3 and 150.4, 8 x 16K 45.2 and 44.1, 256 x 4K (merged
+// in the split kernel) 309 and 302; sessions whose layer fits the L2 the same.
+// Sessions of one split leave no partials and keep the default (256 x 1 000
+// 80.3 and 81.2).
 __device__ __forceinline__ uint64_t copy_policy(bool stream) {
     uint64_t p, q;
     asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
@@ -573,7 +574,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     }
     __syncwarp();
 
-    const uint64_t policy = copy_policy(a.stream != 0);
+    const uint64_t policy = copy_policy(nsplit > 1);
     // Producer step (lane 0): tile k of this warp, in block blk, into slot
     // k % kStages.
     auto issue = [&](int k, int blk) {
@@ -1271,7 +1272,6 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // 32 x 4K -5 % when shorter grids merged too).
     ka.merge_max_splits = ctas >= 8 * sms ? kSplitKernelMerge : 0;
     const bool combine = sub > 1 || (splits > 1 && splits > ka.merge_max_splits);
-    ka.stream = combine;
     cudaError_t e;
     if (sub == 8)
         e = launch_split<1, 8, 8>(c1, map, ka);

@@ -82,7 +82,6 @@ struct DecodeArgs {
     const uint16_t *k_new, *v_new;
     uint16_t *hot;            // pool base, written only when k_new is set
     int32_t pace;             // > 0: a warp's tiles in flight before the previous kernel ends
-    int32_t stream;           // 1: K/V lines are the first to leave the L2
     int32_t inject_extra_tx;  // test hook: extra bytes expected on one tile (0 normally)
     Shape s;
 };
@@ -93,6 +92,7 @@ struct MigArgs {
     uint8_t *img;
     int64_t T_cap;            // image rows per (layer, K|V, kv-head) run
     int32_t t_begin, t_end;   // tokens to move
+    int32_t once;             // set by the launch: lines leave the L2 first
     int32_t *err;
     Shape s;
 };
@@ -117,6 +117,14 @@ struct AppendArgs {
     Shape s;
 };
 
+// An append whose new block ids ride in the launch: logical blocks from ..
+// from + n - 1 of the row, which the kernel writes itself.
+struct AppendInlineArgs {
+    AppendArgs m;             // m.table: the session's device row, written here
+    int32_t from, n;
+    int32_t blocks[kResumeInlineMax];
+};
+
 // One block move between a hot slot and a session image: tokens [t0, t1) of
 // logical block j (all layers, K and V, all kv-heads).
 struct BlockJob {
@@ -133,7 +141,7 @@ struct BlockJobs {
     int64_t table_stride;
     Shape s;
     int32_t n;
-    int32_t pad;
+    int32_t once;             // as in MigArgs
     BlockJob job[kBlockJobsMax];
 };
 
@@ -171,12 +179,12 @@ cudaError_t prepare_kernels();  // per-device function attributes
 cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_sms,
                           cudaStream_t st, bool overlap_previous);
 // max_ctas > 0 caps the migration grids (kv_pool_set_migration_limit).
-cudaError_t launch_unpack(const MigArgs &a, int num_sms, int max_ctas, cudaStream_t st);
-cudaError_t launch_unpack_inline(const ResumeArgs &r, int num_sms, int max_ctas, cudaStream_t st);
-cudaError_t launch_pack(const MigArgs &a, int num_sms, int max_ctas, cudaStream_t st);
-cudaError_t launch_append(const AppendArgs &a, int num_sms, cudaStream_t st);
-cudaError_t launch_block_jobs(const BlockJobs &a, bool pack, int num_sms, int max_ctas,
-                              cudaStream_t st);
+cudaError_t launch_unpack(MigArgs a, int max_ctas, cudaStream_t st);
+cudaError_t launch_unpack_inline(ResumeArgs &r, int max_ctas, cudaStream_t st);
+cudaError_t launch_pack(MigArgs a, int max_ctas, cudaStream_t st);
+cudaError_t launch_append(const AppendArgs &a, cudaStream_t st);
+cudaError_t launch_append_inline(const AppendInlineArgs &r, cudaStream_t st);
+cudaError_t launch_block_jobs(BlockJobs &a, bool pack, int max_ctas, cudaStream_t st);
 cudaError_t launch_table_write(const TableWriteArgs &a, cudaStream_t st);
 cudaError_t launch_gather(const GatherArgs &a, cudaStream_t st);
 

@@ -117,6 +117,7 @@ struct kv_pool {
     std::map<int64_t, int64_t> cold_free;  // offset -> bytes
     int64_t cold_used = 0;
 
+    void *d_slab = nullptr;              // the allocation behind the pointers below
     int32_t *d_tables = nullptr;
     float *d_part_o = nullptr;
     float *d_part_ml = nullptr;
@@ -225,6 +226,31 @@ struct kv_pool {
             if (rc) return rc;
         }
         return KV_OK;
+    }
+
+    // Write n tokens at position s.T; the row gains blocks vals[0 .. fresh_n)
+    // at entry `from`, in the same launch where they fit its parameters.
+    int append_device(int32_t sid, const Session &s, const void *k, const void *v, int32_t n,
+                      const int32_t *vals, int64_t from, int64_t fresh_n, cudaStream_t st) {
+        kvt::AppendInlineArgs r;
+        kvt::AppendArgs &a = r.m;
+        a.k = static_cast<const uint8_t *>(k);
+        a.v = static_cast<const uint8_t *>(v);
+        a.table = d_tables + static_cast<int64_t>(sid) * table_stride;
+        a.hot = static_cast<uint8_t *>(cfg.hot_base);
+        a.pos0 = s.T;
+        a.n = n;
+        a.err = d_err;
+        a.s = shape;
+        if (fresh_n > 0 && fresh_n <= kvt::kResumeInlineMax) {
+            r.from = static_cast<int32_t>(from);
+            r.n = static_cast<int32_t>(fresh_n);
+            std::memcpy(r.blocks, vals, sizeof(int32_t) * fresh_n);
+            return cuda("append launch", [&] { return kvt::launch_append_inline(r, st); });
+        }
+        int rc = fresh_n > 0 ? write_table(sid, vals, from, fresh_n, st) : KV_OK;
+        if (!rc) rc = cuda("append launch", [&] { return kvt::launch_append(a, st); });
+        return rc;
     }
 
     // ---- residency mode -------------------------------------------------
@@ -363,10 +389,10 @@ struct kv_pool {
             a.table_stride = table_stride;
             a.s = shape;
             a.n = static_cast<int32_t>(std::min<size_t>(kvt::kBlockJobsMax, jobs.size() - i));
-            a.pad = 0;
+            a.once = 0;
             std::copy(jobs.begin() + i, jobs.begin() + i + a.n, a.job);
             int rc = cuda(pack ? "pack launch" : "unpack launch",
-                          [&] { return kvt::launch_block_jobs(a, pack, num_sms, mig_ctas, st); });
+                          [&] { return kvt::launch_block_jobs(a, pack, mig_ctas, st); });
             if (rc) return rc;
         }
         return KV_OK;
@@ -380,6 +406,7 @@ struct kv_pool {
         m.T_cap = s.cap;
         m.t_begin = 0;
         m.t_end = 0;
+        m.once = 0;
         m.err = d_err;
         m.s = shape;
         return m;
@@ -466,21 +493,33 @@ int kv_pool_create(const kv_pool_config *cfg, kv_pool **out) {
         p->part_alloc = std::max({p->part_rows, std::min(8 * p->part_rows, 2 * wave),
                                   std::min(2 * p->part_rows, 3 * wave)});
         const int64_t prow = p->part_alloc;
-        int rc = p->cuda("cudaMalloc(tables)", [&] { return cudaMalloc(&p->d_tables, tbl); });
-        if (!rc) rc = p->cuda("cudaMalloc(partials)", [&] {
-            return cudaMalloc(&p->d_part_o, prow * kvt::kHeadDim * sizeof(float));
-        });
-        if (!rc) rc = p->cuda("cudaMalloc(partials)", [&] {
-            return cudaMalloc(&p->d_part_ml, prow * 2 * sizeof(float));
-        });
         // A multi-split call has at most part_rows / Hq layer-batch rows.
         p->counter_count = p->part_rows / c.num_q_heads * c.num_kv_heads;
-        const int64_t cnt = p->counter_count * 4;
-        if (!rc) rc = p->cuda("cudaMalloc(counters)", [&] { return cudaMalloc(&p->d_counters, cnt); });
-        if (!rc) rc = p->cuda("cudaMemset", [&] { return cudaMemset(p->d_counters, 0, cnt); });
-        if (!rc) rc = p->cuda("cudaMalloc(err)", [&] { return cudaMalloc(&p->d_err, 4); });
-        if (!rc) rc = p->cuda("cudaMemset", [&] { return cudaMemset(p->d_err, 0, 4); });
+        // One allocation holds all of it, the words that start at zero last.
+        int64_t bytes = 0;
+        auto place = [&](int64_t n) {
+            const int64_t at = bytes;
+            bytes += (n + 255) / 256 * 256;
+            return at;
+        };
+        const int64_t at_o = place(prow * kvt::kHeadDim * sizeof(float));
+        const int64_t at_ml = place(prow * 2 * sizeof(float));
+        const int64_t at_tables = place(tbl);
+        const int64_t at_counters = place(p->counter_count * 4);
+        const int64_t at_err = place(4);
+        int rc = p->cuda("cudaMalloc(pool metadata)", [&] { return cudaMalloc(&p->d_slab, bytes); });
+        if (!rc) {
+            uint8_t *base = static_cast<uint8_t *>(p->d_slab);
+            p->d_part_o = reinterpret_cast<float *>(base + at_o);
+            p->d_part_ml = reinterpret_cast<float *>(base + at_ml);
+            p->d_tables = reinterpret_cast<int32_t *>(base + at_tables);
+            p->d_counters = reinterpret_cast<int32_t *>(base + at_counters);
+            p->d_err = reinterpret_cast<int32_t *>(base + at_err);
+        }
         if (!rc) rc = p->cuda("cudaMemset", [&] { return cudaMemset(p->d_tables, 0xFF, tbl); });
+        if (!rc) rc = p->cuda("cudaMemset", [&] {
+            return cudaMemset(p->d_counters, 0, bytes - at_counters);
+        });
         if (!rc) rc = p->cuda("kernel attributes", [&] { return kvt::prepare_kernels(); });
         for (int f = 0; !rc && f < kFenceSlots; ++f)
             rc = p->cuda("cudaEventCreate", [&] {
@@ -511,11 +550,7 @@ int kv_pool_destroy(kv_pool *p) {
         }
         for (auto &f : p->fences)
             if (f.ev) cudaEventDestroy(f.ev);
-        cudaFree(p->d_tables);
-        cudaFree(p->d_part_o);
-        cudaFree(p->d_part_ml);
-        cudaFree(p->d_counters);
-        cudaFree(p->d_err);
+        cudaFree(p->d_slab);
     }
     delete p;
     return KV_OK;
@@ -640,20 +675,8 @@ static int lru_append(kv_pool *p, int32_t sid, const void *k, const void *v, int
         rc = p->run_jobs({p->fetch_job(sid, static_cast<int32_t>(tail), got[0], 0,
                                        p->tokens_in_block(*s, tail))}, false, st);
     }
-    if (!rc && fresh_n > 0)
-        rc = p->write_table(sid, got.data() + (refetch ? 1 : 0), have, fresh_n, st);
-    if (!rc) {
-        kvt::AppendArgs a;
-        a.k = static_cast<const uint8_t *>(k);
-        a.v = static_cast<const uint8_t *>(v);
-        a.table = p->d_tables + static_cast<int64_t>(sid) * p->table_stride;
-        a.hot = static_cast<uint8_t *>(p->cfg.hot_base);
-        a.pos0 = s->T;
-        a.n = n;
-        a.err = p->d_err;
-        a.s = p->shape;
-        rc = p->cuda("append launch", [&] { return kvt::launch_append(a, p->num_sms, st); });
-    }
+    if (!rc)
+        rc = p->append_device(sid, *s, k, v, n, got.data() + (refetch ? 1 : 0), have, fresh_n, st);
     if (!rc) rc = p->cuda("cudaEventRecord", [&] { return cudaEventRecord(s->appended, st); });
     if (rc) return rc;   // host state untouched
 
@@ -840,19 +863,7 @@ int session_append(kv_pool *p, int32_t sid, const void *k, const void *v, int32_
     if (!rc && s->ready_recorded)
         rc = p->cuda("cudaStreamWaitEvent", [&] { return cudaStreamWaitEvent(st, s->ready, 0); });
     if (!rc && need > 0) rc = p->wait_fences(fresh.data(), fresh.size(), st);
-    if (!rc && need > 0) rc = p->write_table(sid, fresh.data(), have, need, st);
-    if (!rc) {
-        kvt::AppendArgs a;
-        a.k = static_cast<const uint8_t *>(k);
-        a.v = static_cast<const uint8_t *>(v);
-        a.table = p->d_tables + static_cast<int64_t>(sid) * p->table_stride;
-        a.hot = static_cast<uint8_t *>(p->cfg.hot_base);
-        a.pos0 = s->T;
-        a.n = n;
-        a.err = p->d_err;
-        a.s = p->shape;
-        rc = p->cuda("append launch", [&] { return kvt::launch_append(a, p->num_sms, st); });
-    }
+    if (!rc) rc = p->append_device(sid, *s, k, v, n, fresh.data(), have, need, st);
     if (!rc)
         rc = p->cuda("cudaEventRecord", [&] { return cudaEventRecord(s->appended, st); });
     if (rc) return rc;   // host state untouched
@@ -979,7 +990,7 @@ int session_pause(kv_pool *p, int32_t sid, kv_stream_t stream_) {
         kvt::MigArgs m = p->mig_args(sid, *s);
         m.t_begin = static_cast<int32_t>(t0);
         m.t_end = static_cast<int32_t>(t1);
-        rc = p->cuda("pack launch", [&] { return kvt::launch_pack(m, p->num_sms, p->mig_ctas, st); });
+        rc = p->cuda("pack launch", [&] { return kvt::launch_pack(m, p->mig_ctas, st); });
     }
     if (!rc) rc = p->cuda("cudaEventRecord", [&] { return cudaEventRecord(p->fences[f].ev, st); });
     if (rc) return rc;
@@ -1041,7 +1052,7 @@ int session_resume(kv_pool *p, int32_t sid, kv_stream_t stream_) {
         r.pad = 0;
         std::memcpy(r.blocks, fresh.data(), sizeof(int32_t) * need);
         rc = p->cuda("unpack launch",
-                     [&] { return kvt::launch_unpack_inline(r, p->num_sms, p->mig_ctas, st); });
+                     [&] { return kvt::launch_unpack_inline(r, p->mig_ctas, st); });
     } else if (!rc) {
         rc = p->write_table(sid, fresh.data(), 0, need, st);
         if (!rc) {
@@ -1049,7 +1060,7 @@ int session_resume(kv_pool *p, int32_t sid, kv_stream_t stream_) {
             m.t_begin = 0;
             m.t_end = static_cast<int32_t>(s->T);
             rc = p->cuda("unpack launch",
-                         [&] { return kvt::launch_unpack(m, p->num_sms, p->mig_ctas, st); });
+                         [&] { return kvt::launch_unpack(m, p->mig_ctas, st); });
         }
     }
     if (!rc) rc = p->cuda("cudaEventRecord", [&] { return cudaEventRecord(s->ready, st); });
