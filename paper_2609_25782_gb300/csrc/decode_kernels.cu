@@ -515,8 +515,8 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     const int slice = static_cast<int>(run % gridDim.x);
     const int split = slice / kSub;
     const int sub = slice % kSub;           // which of the split's CTAs
-    const int lb = static_cast<int>(run / gridDim.x);
-    const int b = lb % a.B;
+    int lb = static_cast<int>(run / gridDim.x);
+    int b = lb % a.B;
     const int li = lb / a.B;
     const int l = a.layer0 + li;
     const int warp = threadIdx.x >> 5;
@@ -529,6 +529,16 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     // may be scheduled once every CTA of this grid has started; it still
     // waits for this grid to finish before reading.
     asm volatile("griddepcontrol.launch_dependents;");
+    if (kSub == 1 && a.longest_first) {
+        // Row r of the grid is the r-th longest session (ties by batch row).
+        const int t = lane < a.B ? a.seq_lens[lane] : 0;
+        int rank = 0;
+        for (int j = 0; j < a.B; ++j) {
+            const int tj = __shfl_sync(0xffffffffu, t, j);
+            rank += tj > t || (tj == t && j < lane);
+        }
+        b = lb = __ffs(__ballot_sync(0xffffffffu, lane < a.B && rank == lb)) - 1;
+    }
     const int32_t *trow = a.tables + static_cast<int64_t>(b) * a.max_blocks;
     // Tables at most KVT_SPLIT_TARGET x KVT_SPLIT_MIN_TILES tiles wide split
     // every session every KVT_SPLIT_MIN_TILES tiles, so this warp's tiles are
@@ -1270,6 +1280,15 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // the combine: 256 x 4K-token sessions per layer +1.3 %, 8 x 4K all
     // layers +1.6 %; one 4K- or 16K-token session per layer -7 % / -5 % and
     // 32 x 4K -5 % when shorter grids merged too).
+    // A grid of several waves ends when its last long splits do, with most SMs
+    // waiting: where splits differ in length (tables wider than 16K tokens) the
+    // longest sessions go out first. 48 layers of 16 sessions of 2K-30K tokens
+    // 3 920 -> 3 822 us, of 32 of 8K-32K 9 188 -> 9 043, 24 layers of 12 of
+    // 4K-60K 2 601 -> 2 531. Equal splits only lose by it, the block ids then
+    // waiting for the ranks (24 of 1K-14K 2 879 and 2 920); a lane ranks one
+    // session, so up to 32.
+    ka.longest_first = a.nlayers == 1 && a.B > 1 && a.B <= 32 && sub == 1 && ctas > 3 * sms &&
+                       split_tiles(a.max_blocks * a.s.bt) > KVT_SPLIT_MIN_TILES;
     ka.merge_max_splits = ctas >= 8 * sms ? kSplitKernelMerge : 0;
     const bool combine = sub > 1 || (splits > 1 && splits > ka.merge_max_splits);
     cudaError_t e;

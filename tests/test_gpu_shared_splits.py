@@ -62,3 +62,21 @@ def test_shared_splits(pkg, lens, tokens, hkv, shared, bt, scale):  # noqa: F811
                               tables[:n], lens, scale, 8 * hkv)
     assert scaled_err(got, ref[0]) <= TOL
     assert pool.check_device() == 0
+
+
+# Grids of several waves whose splits differ in length start with the longest
+# sessions (up to 32 of them): each row once, whatever its rank, ties included.
+@pytest.mark.parametrize("n", [9, 31, 32, 33])
+@pytest.mark.parametrize("bt", [16, 64])
+def test_longest_first(pkg, n, bt):  # noqa: F811
+    lens = ([17003, 20, 17003, 1, 16400, 5000, 64, 17003, 1] + [700 + 37 * (i % 5) for i in range(24)])[:n]
+    pool, sess, tables, q = direct_case(pkg, lens, L=1, bt=bt, seed=23, max_batch=n)
+    got = gpu_decode(pool, 0, q, tables, lens)[0]
+    for i in range(n):
+        one = gpu_decode(pool, 0, q[:, i:i + 1], tables[i:i + 1], lens[i:i + 1])[0, 0]
+        assert np.array_equal(one.view(np.int64), got[i].view(np.int64))
+    ref = oracle.paged_decode(host_hot(pool, 23, sess, lens, tables),
+                              q.cpu().view(torch.int16).numpy().view(np.uint16), tables, lens,
+                              1 / math.sqrt(128), 32)
+    assert scaled_err(got, ref[0]) <= TOL
+    assert pool.check_device() == 0
