@@ -35,7 +35,10 @@ constexpr int kMigChunkTokens = 16;     // tokens per migration item (divides bt
 constexpr int kMigUnroll = 4;           // 32-byte loads in flight per lane
 static_assert(kMigChunkTokens * kRowBytes == 32 * 32 * kMigUnroll, "one round moves a chunk");
 constexpr int64_t kOnceBytes = int64_t(32) << 20;   // a quarter of the L2
-constexpr int kAppendUnroll = 4;        // 16-byte loads in flight per lane
+constexpr int kAppendRows = 16;         // head rows an append warp moves
+__host__ __device__ constexpr int append_group(int Hkv) {   // tokens that make them up
+    return Hkv * 2 >= kAppendRows ? 1 : kAppendRows / (2 * Hkv);
+}
 
 struct alignas(32) Row32 {
     uint32_t w[8];
@@ -173,49 +176,67 @@ __global__ void __launch_bounds__(256) block_jobs_kernel(const __grid_constant__
     }
 }
 
-// K5: one warp per (layer, token): the token's K and V rows for all kv-heads
-// are 2 x Hkv*256 contiguous bytes in the source; each 256-byte head row goes
-// to its (layer, K|V, head) run of the tail block.
-// One warp per (layer, token) item, items layer-major so that consecutive
-// warps read k and v sequentially. A lane issues all of its 16-byte loads of
-// the item (K and V rows of every kv-head) before its first store.
+// K5: one warp per (layer, group of tokens). A token's K (or V) rows for all
+// kv-heads are Hkv*256 contiguous bytes in the source, and so are the next
+// token's; each 256-byte head row goes to its (layer, K|V, head) run of the
+// token's block, beside the token before. A group is the tokens that make up 16
+// head rows (4 KiB, one token of 8 kv-heads, four of 2), so that a warp moves as
+// much whatever the shape, in one round of 16-byte loads, eight per lane, half a
+// warp per row (k and v need be aligned to no more). Items are layer-major so that
+// consecutive warps read k and v sequentially. Bound by HBM; one token per warp
+// in its place: a turn of 16 000 tokens of 2 kv-heads, 16 layers, appended and
+// packed, 180 -> 155 us.
 // block_of(j) gives logical block j's slot.
 template <typename BlockOf>
 __device__ __forceinline__ void append_tokens(const AppendArgs &a, BlockOf block_of) {
     const Shape sh = a.s;
-    const int items = sh.L * a.n;
+    const int group = append_group(sh.Hkv);
+    const int groups = (a.n + group - 1) / group;
+    const int items = sh.L * groups;
     const int lane = threadIdx.x & 31;
-    const int units = sh.Hkv * (kRowBytes / 16);   // 16-byte units per K (or V) token
+    const int c = lane & 15;                         // 16-byte unit of a row
+    const int64_t run_bytes = static_cast<int64_t>(sh.bt) * kRowBytes;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += nwarps) {
-        const int l = it / a.n;
-        const int i = it - l * a.n;
+        const int l = it / groups;
+        const int i = (it - l * groups) * group;
+        const int rows = min(group, a.n - i) * sh.Hkv;   // of K, and again of V
+        const int64_t src_off = (static_cast<int64_t>(l) * a.n + i) * sh.Hkv * kRowBytes;
+        const uint4 *ks = reinterpret_cast<const uint4 *>(a.k + src_off) + c;
+        const uint4 *vs = reinterpret_cast<const uint4 *>(a.v + src_off) + c;
+        uint4 v[kAppendRows / 2];
+#pragma unroll
+        for (int k = 0; k < kAppendRows / 2; ++k) {
+            const int r = 2 * k + (lane >> 4);
+            if (r < 2 * rows) v[k] = ld_stream(r < rows ? ks + r * 16 : vs + (r - rows) * 16);
+        }
+        // The group lies in one block, or in two.
         const int64_t t = a.pos0 + i;
-        const int64_t src_off = static_cast<int64_t>(it) * sh.Hkv * kRowBytes;
-        const uint4 *ks = reinterpret_cast<const uint4 *>(a.k + src_off);
-        const uint4 *vs = reinterpret_cast<const uint4 *>(a.v + src_off);
-        const int blk = block_of(static_cast<int>(t / sh.bt));
-        const bool ok = blk >= 0 && blk < sh.num_blocks;
-        if (!ok && lane == 0) atomicOr(a.err, kErrBadBlock);
-        // Unit u = (kv * Hkv + g) * 16 + c lands in run (kv, g), row `slot`.
-        const int slot = static_cast<int>(t % sh.bt);
-        uint8_t *base = a.hot + ((static_cast<int64_t>(ok ? blk : 0) * sh.L + l) * 2 * sh.Hkv *
-                                     sh.bt + slot) * kRowBytes;
-        const int64_t run_bytes = static_cast<int64_t>(sh.bt) * kRowBytes;
-        for (int u0 = 0; u0 < 2 * units; u0 += 32 * kAppendUnroll) {
-            uint4 v[kAppendUnroll];
+        const int j = static_cast<int>(t / sh.bt);
+        const int slot0 = static_cast<int>(t - static_cast<int64_t>(j) * sh.bt);
+        uint8_t *base[2];
 #pragma unroll
-            for (int k = 0; k < kAppendUnroll; ++k) {
-                const int u = u0 + k * 32 + lane;
-                if (u < 2 * units) v[k] = ld_stream(u < units ? ks + u : vs + (u - units));
-            }
-            if (!ok) continue;
+        for (int s = 0; s < 2; ++s) {
+            const bool used = s == 0 || slot0 + rows / sh.Hkv > sh.bt;
+            const int blk = used ? block_of(j + s) : -1;
+            const bool ok = blk >= 0 && blk < sh.num_blocks;
+            if (used && !ok && lane == 0) atomicOr(a.err, kErrBadBlock);
+            base[s] = ok ? a.hot + (static_cast<int64_t>(blk) * sh.L + l) * 2 * sh.Hkv * run_bytes + c * 16
+                         : nullptr;
+        }
 #pragma unroll
-            for (int k = 0; k < kAppendUnroll; ++k) {
-                const int u = u0 + k * 32 + lane;
-                if (u < 2 * units)
-                    reinterpret_cast<uint4 *>(base + (u >> 4) * run_bytes)[u & 15] = v[k];
-            }
+        for (int k = 0; k < kAppendRows / 2; ++k) {
+            const int r = 2 * k + (lane >> 4);
+            if (r >= 2 * rows) continue;
+            const int kv = r >= rows;
+            const int w = r - kv * rows;             // token and head of the row
+            const int ti = w / sh.Hkv;
+            const int slot = slot0 + ti;
+            const int next = slot >= sh.bt;
+            uint8_t *to = next ? base[1] : base[0];
+            if (to != nullptr)
+                *reinterpret_cast<uint4 *>(to + (kv * sh.Hkv + (w - ti * sh.Hkv)) * run_bytes +
+                                           (slot - next * sh.bt) * kRowBytes) = v[k];
         }
     }
 }
@@ -227,7 +248,7 @@ __global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
 // An append whose new block ids ride in the launch: the grid also writes them
 // to the session's table row (read by later work only), which saves the
 // table-write launch in front of it: a turn of 1 536 tokens, appended and
-// packed, 98.5 -> KVT_TURN us.
+// packed, 98.0 -> 94.3 us.
 __global__ void __launch_bounds__(256) append_inline_kernel(const __grid_constant__ AppendInlineArgs r) {
     const int nthreads = gridDim.x * blockDim.x;
     int32_t *row = const_cast<int32_t *>(r.m.table);   // the pool's own row: writable
@@ -299,14 +320,19 @@ cudaError_t launch_pack(MigArgs a, int max_ctas, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+static int64_t append_items(const AppendArgs &a) {
+    const int group = append_group(a.s.Hkv);
+    return static_cast<int64_t>(a.s.L) * ((a.n + group - 1) / group);
+}
+
 cudaError_t launch_append(const AppendArgs &a, cudaStream_t st) {
-    append_kernel<<<item_grid(static_cast<int64_t>(a.s.L) * a.n, 0), 256, 0, st>>>(a);
+    append_kernel<<<item_grid(append_items(a), 0), 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_append_inline(const AppendInlineArgs &r, cudaStream_t st) {
     if (r.n < 1 || r.n > kResumeInlineMax) return cudaErrorInvalidValue;
-    append_inline_kernel<<<item_grid(static_cast<int64_t>(r.m.s.L) * r.m.n, 0), 256, 0, st>>>(r);
+    append_inline_kernel<<<item_grid(append_items(r.m), 0), 256, 0, st>>>(r);
     return cudaGetLastError();
 }
 

@@ -521,10 +521,6 @@ int kv_pool_create(const kv_pool_config *cfg, kv_pool **out) {
             return cudaMemset(p->d_counters, 0, bytes - at_counters);
         });
         if (!rc) rc = p->cuda("kernel attributes", [&] { return kvt::prepare_kernels(); });
-        for (int f = 0; !rc && f < kFenceSlots; ++f)
-            rc = p->cuda("cudaEventCreate", [&] {
-                return cudaEventCreateWithFlags(&p->fences[f].ev, cudaEventDisableTiming);
-            });
         if (rc) return bail(rc);
         const char *why = nullptr;
         if (!kvt::encode_hot_tensor_map(&p->tmap, c.hot_base, rows,
@@ -978,8 +974,8 @@ int session_pause(kv_pool *p, int32_t sid, kv_stream_t stream_) {
     // Fence slot that will mark the freed blocks; its previous pack must be
     // complete before the slot is re-recorded.
     const int f = p->next_fence;
-    int rc = KV_OK;
-    if (p->fences[f].gen != 0)
+    int rc = ensure_event(p, &p->fences[f].ev);
+    if (!rc && p->fences[f].gen != 0)
         rc = p->cuda("cudaEventSynchronize", [&] { return cudaEventSynchronize(p->fences[f].ev); });
     if (!rc && s->appended_recorded)
         rc = p->cuda("cudaStreamWaitEvent", [&] { return cudaStreamWaitEvent(st, s->appended, 0); });

@@ -18,13 +18,14 @@ def device_row(pool, sid):
 
 @pytest.mark.parametrize("bt", [16, 64])
 @pytest.mark.parametrize("lru", [False, True])
+@pytest.mark.parametrize("hkv", [1, 2, 3, 8])
 # 2 048 blocks of 16 tokens fill the launch; one more goes through a table write
 @pytest.mark.parametrize("parts", [[1], [16], [17, 47, 1], [5, 32768], [7, 32769 + 16], [64, 1, 63]])
-def test_append_rows(cuda_dev, bt, lru, parts):
+def test_append_rows(cuda_dev, bt, lru, hkv, parts):
     import __graft_entry__
     __graft_entry__.build()
     from paper_2609_25782_gb300 import Pool
-    L, hkv, d = 2, 2, 128
+    L, d = 2, 128
     total = sum(parts)
     nb = -(-total // bt) + 3
     cap = total * L * 2 * hkv * d * 2 + 256
