@@ -57,8 +57,8 @@ constexpr int kHalfBytes = 2048;           // 16 rows x 128 B (64 dims)
 //   <4 warps, 3 slots, 1>           2 CTAs per SM
 //   <8 warps, 3 slots, 1>           1 CTA per SM: one accumulator per warp,
 //                                   twice the warps per SM
-//   <8 / kSub warps, slots, kSub>   a split shared by kSub = 2, 4 or 8 CTAs,
-//                                   one accumulator per warp: grids of up to
+//   <8 / kSub warps, slots, kSub>   a split shared by kSub = 2 or 8 CTAs, one
+//                                   accumulator per warp: grids of up to
 //                                   three CTAs per SM once shared
 constexpr int kAccs = 8;
 // Lazy softmax maximum: the reference moves when a logit exceeds it by more
@@ -272,7 +272,7 @@ __device__ __forceinline__ void join_accs(float (&m)[kN], float (&l)[kN], float4
 }
 
 // Partial rows per split of a grid whose splits are shared by `sub` CTAs: one
-// per half where each CTA holds one, else one per accumulator.
+// per half where each of two CTAs holds one, one per accumulator for eight.
 __host__ __device__ constexpr int parts_per_split(int sub) {
     return sub <= 2 ? sub : kAccs;
 }
@@ -1175,7 +1175,6 @@ cudaError_t prepare_kernels() {
     if (e == cudaSuccess) e = prepare_split<4, 6, 2>();
     if (e == cudaSuccess) e = prepare_split<4, 3, 2>();
     if (e == cudaSuccess) e = prepare_split<4, 2, 2>();
-    if (e == cudaSuccess) e = prepare_split<2, 6, 4>();
     if (e == cudaSuccess) e = prepare_split<1, 8, 8>();
     return e;
 }
@@ -1218,8 +1217,9 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // it before the previous call ends, and is gone sooner, so the next call's
     // CTAs start their copies sooner. The combine reads 2 or 8 states per split
     // instead of one. us per layer, unshared and shared:
-    //   8 or 4 CTAs, at most one per SM: 1 x 3 001 8.04 and 5.36, 1 x 8K 8.51
-    //     and 6.74, 4 x 1 280 8.26 and 6.17
+    //   8 (one warp each, its ring the whole of a 64-tile split), at most two
+    //     per SM: 1 x 3 001 8.04 and 5.14, 1 x 8K 8.51 and 5.70, 4 x 1 280 8.26
+    //     and 5.10 (shared by 4 of two warps, one per SM: 6.85 and 6.51)
     //   2, at most one per SM: 1 x 16 391 9.97 and 8.72 (two CTAs per SM with
     //     half the ring 10.0, four of a shorter split 10.6)
     //   2, two per SM: 8 x 4K 13.1 and 12.4, 2 x 16K 13.3 and 12.6, 5 x 5K 11.6
@@ -1242,10 +1242,8 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     int sub = 1;
     int per_sm = 1;   // of a shared grid
     if (splits > 1) {
-        if (!wide && fits(8, 1))
+        if (!wide && fits(8, 2))
             sub = 8;
-        else if (!wide && fits(4, 1))
-            sub = 4;
         else if (fits(2, 1))
             sub = 2;
         else if (fits(2, 2))
@@ -1261,7 +1259,7 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // still keep HBM busy and the chain behind them is shorter. us per layer,
     // unpaced and paced: one session of 16 391 tokens 8.64 and 7.98, 32K 13.6
     // and 12.7; 8 x 4K 15.0 and 13.2, 12 x 2K 12.1 and 11.4; 4 x 16K 24.1 and
-    // 23.1. Rings that cover a whole split (4 or 8 CTAs per split) showed no
+    // 23.1. Rings that cover a whole split (8 CTAs per split) showed no
     // difference, and in grids of more than one wave the later CTAs lose by it
     // (8 x 16K 44.4 and 45.1). Calls without a combine (40 x 1 000 16.0 and
     // 16.9) and unshared long splits (1 x 100K) take no part.
@@ -1294,8 +1292,6 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     cudaError_t e;
     if (sub == 8)
         e = launch_split<1, 8, 8>(c1, map, ka);
-    else if (sub == 4)
-        e = launch_split<2, 6, 4>(c1, map, ka);
     else if (sub == 2 && per_sm == 1)
         e = launch_split<4, 6, 2>(c1, map, ka);
     else if (sub == 2 && per_sm == 2)
@@ -1328,7 +1324,7 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     if (wide)
         return sub == 2 ? cudaLaunchKernelEx(&c2, decode_combine_kernel<2, 8>, ka)
                         : cudaLaunchKernelEx(&c2, decode_combine_kernel<1, 16>, ka);
-    if (sub > 2) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<8>, ka);
+    if (sub == 8) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<8>, ka);
     return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<2>, ka);
 }
 

@@ -486,9 +486,9 @@ int kv_pool_create(const kv_pool_config *cfg, kv_pool **out) {
             return bail(fail(KV_ERR_CUDA, "cudaSetDevice failed"));
         cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, c.device);
         const int64_t tbl = static_cast<int64_t>(c.max_sessions) * p->table_stride * 4;
-        // Small grids share a split among 8 or 4 CTAs, at most one per SM, and
-        // leave 8 partial rows of it, or among 2, at most three per SM, and
-        // leave 2 (launch_decode).
+        // Small grids share a split among 8 CTAs, at most two per SM, and leave
+        // 8 partial rows of it, or among 2, at most three per SM, and leave 2
+        // (launch_decode).
         const int64_t wave = static_cast<int64_t>(p->num_sms) * (c.num_q_heads / c.num_kv_heads);
         p->part_alloc = std::max({p->part_rows, std::min(8 * p->part_rows, 2 * wave),
                                   std::min(2 * p->part_rows, 3 * wave)});
