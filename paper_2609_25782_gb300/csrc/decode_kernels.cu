@@ -480,8 +480,8 @@ __device__ __forceinline__ void merge_states(const DecodeArgs &a, int64_t row_ba
 //
 // Large grids are bound by HBM. A small one (a layer of one or a few
 // sessions) is a chain of latencies: the previous call's end, q, a warp's
-// tiles one after another (0.36 us each; 0.16 us in a batch of 4, whose 64
-// mma.sync alone take 0.27 us of one tensor pipe), the merge, the combine.
+// tiles one after another (0.36 us each; in a batch of 4, whose 64 mma.sync
+// alone take 0.27 us of one tensor pipe, 0.62 us), the merge, the combine.
 // It also runs every instruction once or twice, so its code has to stay in
 // the instruction cache (straight-line code of over about 32 KB is fetched at
 // 2.7 cycles an instruction): loops that are not on the tile path stay rolled
@@ -1268,16 +1268,6 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
         ka.pace = per_sm == 1 ? 2 : 1;
     else if (overlap_previous && sub == 1 && splits > 1 && !wide && ctas <= 2 * sms)
         ka.pace = 1;
-
-    // Which sessions the split kernel merges itself (the bits are the same
-    // either way): those of up to kSplitKernelMerge splits, in grids of at
-    // least 8 CTAs per SM. There, many groups finish at different times and
-    // their merges spread over the grid. In shorter grids each CTA's arrival
-    // (an atomic round trip holding its SM slot) and the tail merges cost more
-    // than the combine launch (measured on GB300 against merging everything in
-    // the combine: 256 x 4K-token sessions per layer +1.3 %, 8 x 4K all
-    // layers +1.6 %; one 4K- or 16K-token session per layer -7 % / -5 % and
-    // 32 x 4K -5 % when shorter grids merged too).
     // A grid of several waves ends when its last long splits do, with most SMs
     // waiting: where splits differ in length (tables wider than 16K tokens) the
     // longest sessions go out first. 48 layers of 16 sessions of 2K-30K tokens
@@ -1287,6 +1277,15 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // session, so up to 32.
     ka.longest_first = a.nlayers == 1 && a.B > 1 && a.B <= 32 && sub == 1 && ctas > 3 * sms &&
                        split_tiles(a.max_blocks * a.s.bt) > KVT_SPLIT_MIN_TILES;
+    // Which sessions the split kernel merges itself (the bits are the same
+    // either way): those of up to kSplitKernelMerge splits, in grids of at
+    // least 8 CTAs per SM. There, many groups finish at different times and
+    // their merges spread over the grid. In shorter grids each CTA's arrival
+    // (an atomic round trip holding its SM slot) and the tail merges cost more
+    // than the combine launch (measured on GB300 against merging everything in
+    // the combine: 256 x 4K-token sessions per layer +1.3 %, 8 x 4K all
+    // layers +1.6 %; one 4K- or 16K-token session per layer -7 % / -5 % and
+    // 32 x 4K -5 % when shorter grids merged too).
     ka.merge_max_splits = ctas >= 8 * sms ? kSplitKernelMerge : 0;
     const bool combine = sub > 1 || (splits > 1 && splits > ka.merge_max_splits);
     cudaError_t e;
