@@ -480,9 +480,12 @@ __device__ __forceinline__ void merge_states(const DecodeArgs &a, int64_t row_ba
 //
 // Large grids are bound by HBM. A small one (a layer of one or a few
 // sessions) is a chain of latencies: the previous call's end, q, a warp's
-// tiles one after another (0.36 us each; in a batch of 4, whose 64 mma.sync
-// alone take 0.27 us of one tensor pipe, 0.62 us), the merge, the combine.
-// It also runs every instruction once or twice, so its code has to stay in
+// tiles one after another (0.36 us each), the merge, the combine. So a warp of
+// a shared split takes tiles that have landed in twos (tile_batch): 48 layers of
+// one session of 3 001 tokens with peaked scores 295 us in fours that went back
+// to single tiles where a maximum moved, 263 in fours, 258 in twos; of 16 391
+// tokens 372, 377 and 367.
+// Such a call also runs every instruction once or twice, so its code has to stay in
 // the instruction cache (straight-line code of over about 32 KB is fetched at
 // 2.7 cycles an instruction): loops that are not on the tile path stay rolled
 // and the rare steps are in one place.
@@ -778,9 +781,9 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     // last, into the one accumulator of a warp: the values of one_tile on each
     // in turn, with the score products side by side and the next fragments on
     // their way while a step's products run. The weights follow together too,
-    // unless a tile after the first of all moves the maximum: then nothing has
-    // been added yet and the caller takes the tiles one by one (false).
-    auto tile_batch = [&](auto n_const, int k, AccState &s) -> bool {
+    // unless a tile after the first of all moves the maximum (peaked scores):
+    // then the tiles go one by one from their scores on, in a rolled loop.
+    auto tile_batch = [&](auto n_const, int k, AccState &s) {
         constexpr int kN = decltype(n_const)::value;
         float sa[kN][4], sb[kN][4], x[kN][4];
 #pragma unroll
@@ -815,19 +818,35 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         bool grow = false;
 #pragma unroll
         for (int i = 0; i < kN; ++i) grow |= grows(x[i], s);
-        if (__any_sync(0xffffffffu, grow)) return false;
-        uint32_t pb[kN][2];
+        if (__any_sync(0xffffffffu, grow)) {
+#pragma unroll 1
+            for (int i = 0; i < kN; ++i) {
+                float y[4];
 #pragma unroll
-        for (int i = 0; i < kN; ++i) weights(x[i], s, pb[i][0], pb[i][1]);
+                for (int j = 0; j < 4; ++j) {
+                    y[j] = x[0][j];
 #pragma unroll
-        for (int i = 0; i < kN; ++i) {
-            if (i + 1 < kN) load_values(slot_of(k + i + 1), vf[(i + 1) & 1]);
-            add_values(vf[i & 1], s, pb[i][0], pb[i][1]);
+                    for (int t = 1; t < kN; ++t) y[j] = i == t ? x[t][j] : y[j];
+                }
+                if (__any_sync(0xffffffffu, grows(y, s))) move_max(y, s);
+                uint32_t pb0, pb1;
+                weights(y, s, pb0, pb1);
+                load_values(slot_of(k + i), vf[0]);
+                add_values(vf[0], s, pb0, pb1);
+            }
+        } else {
+            uint32_t pb[kN][2];
+#pragma unroll
+            for (int i = 0; i < kN; ++i) weights(x[i], s, pb[i][0], pb[i][1]);
+#pragma unroll
+            for (int i = 0; i < kN; ++i) {
+                if (i + 1 < kN) load_values(slot_of(k + i + 1), vf[(i + 1) & 1]);
+                add_values(vf[i & 1], s, pb[i][0], pb[i][1]);
+            }
         }
         __syncwarp();
 #pragma unroll 1
         for (int i = 0; i < kN; ++i) refill(k + i);
-        return true;
     };
 
     if constexpr (kA == 2) {
@@ -853,13 +872,12 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
             }
         }
     } else {
-        constexpr int kBatch = kStages >= 4 ? 4 : 2;
+        constexpr int kBatch = 2;
         // The warp's tiles before the session's last one need no length mask.
         const int plain = tile_base(my_tiles - 1) + kTileTokens >= T ? my_tiles - 1 : my_tiles;
-        int single = 0;   // tiles up to here go one by one
 #pragma unroll 1
         for (int k = 0; k < my_tiles;) {
-            bool batch = k >= single && k + kBatch <= plain;
+            bool batch = k + kBatch <= plain;
             if (batch) {
 #pragma unroll
                 for (int i = 0; i < kBatch; ++i)
@@ -867,11 +885,9 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
                 batch = __all_sync(0xffffffffu, batch);
             }
             if (batch) {
-                if (tile_batch(std::integral_constant<int, kBatch>{}, k, acc_state[0])) {
-                    k += kBatch;
-                    continue;
-                }
-                single = k + kBatch;
+                tile_batch(std::integral_constant<int, kBatch>{}, k, acc_state[0]);
+                k += kBatch;
+                continue;
             }
             if (!one_tile(k, acc_state[0])) {
                 fail_k = k;
