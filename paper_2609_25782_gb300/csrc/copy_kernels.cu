@@ -20,19 +20,24 @@
 namespace kvt {
 namespace {
 
-// Migration copy shape: one warp per 16-token chunk of a run (4 KiB on both
-// sides), moved by one round of 32-byte loads, four per lane, and stores. Bound
+// Migration copy shape: one warp per 8-token chunk of a run (2 KiB on both
+// sides), moved by one round of 32-byte loads, two per lane, and stores. Bound
 // by HBM. The warps are not reused: a grid-stride loop over 32 CTAs per SM moved
 // three sessions of 20K-30K tokens in 2.26 ms, one warp per chunk in 2.19 ms
-// (its 16-byte predecessor in 2.31 ms, 1.00 of the copy bandwidth).
+// (its 16-byte predecessor in 2.31 ms, 1.00 of the copy bandwidth). Four loads
+// per lane over 16 tokens need 48 registers, so five CTAs an SM instead of
+// six, and a move of 29 MB ends with a second wave of a few CTAs: two resumes of
+// 892 tokens, 16 layers, 28.4 us, now 26.1 (27.6 with 16-byte loads); of 1 000
+// 29.0 and 27.5; of 24K, 48 layers, 1 339 and 1 335; three of 892 in a row 80.3
+// and 82.2 (82.2). Held to 40 registers they spill (31.5).
 // Moves larger than kOnceBytes touch image and blocks once and let both leave
 // the L2 first, which leaves room for what others keep there: of a turn of
 // 1 536 tokens, appended and then packed, the pack finds most of the appended
 // blocks in the L2 (96.1 -> 87.4 us with both hints, 94.4 with one of them).
 // Smaller ones may be used again while they are there (two resumes of 300
 // tokens 26.4 us, 28.0 with the hints).
-constexpr int kMigChunkTokens = 16;     // tokens per migration item (divides bt)
-constexpr int kMigUnroll = 4;           // 32-byte loads in flight per lane
+constexpr int kMigChunkTokens = 8;      // tokens per migration item (divides bt)
+constexpr int kMigUnroll = 2;           // 32-byte loads in flight per lane
 static_assert(kMigChunkTokens * kRowBytes == 32 * 32 * kMigUnroll, "one round moves a chunk");
 constexpr int64_t kOnceBytes = int64_t(32) << 20;   // a quarter of the L2
 constexpr int kAppendRows = 16;         // head rows an append warp moves
@@ -101,8 +106,8 @@ template <bool kPack, typename BlockOf>
 __device__ __forceinline__ void migrate_runs(const MigArgs &a, BlockOf block_of) {
     const Shape sh = a.s;
     const int runs = sh.L * 2 * sh.Hkv;
-    // Items are 16-token chunks of a run, so a 64-token block gives four
-    // warps the parallelism a 16-token block gives one.
+    // Items are chunks of a run, so a 64-token block is as many warps' work as
+    // four of 16 tokens.
     const int q0 = a.t_begin / kMigChunkTokens;
     const int q1 = (a.t_end + kMigChunkTokens - 1) / kMigChunkTokens;
     const int nq = q1 - q0;
@@ -149,7 +154,7 @@ template <bool kPack>
 __global__ void __launch_bounds__(256) block_jobs_kernel(const __grid_constant__ BlockJobs a) {
     const Shape sh = a.s;
     const int runs = sh.L * 2 * sh.Hkv;
-    const int cpb = sh.bt / kMigChunkTokens;      // 16-token chunks per block
+    const int cpb = sh.bt / kMigChunkTokens;      // chunks per block
     const int items = a.n * runs * cpb;
     const int lane = threadIdx.x & 31;
     const uint64_t policy = move_policy(a.once);
