@@ -55,6 +55,7 @@ constexpr int kHalfBytes = 2048;           // 16 rows x 128 B (64 dims)
 //                                   and w + 4 and alternates between them, so
 //                                   consecutive tiles of a warp are independent
 //   <4 warps, 3 slots, 1>           2 CTAs per SM
+//   the same two, true              their CTAs take the longest sessions first
 //   <8 warps, 3 slots, 1>           1 CTA per SM: one accumulator per warp,
 //                                   twice the warps per SM
 //   <8 / kSub warps, slots, kSub>   a split shared by kSub = 2 or 8 CTAs, one
@@ -496,7 +497,7 @@ struct AccState {
     float o[8][4];  // O^T fragments
 };
 
-template <int kWarps, int kStages, int kSub>
+template <int kWarps, int kStages, int kSub, bool kByLength = false>
 __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kStages == 2 ? 3 : kStages == 3 ? 2 : 1)
     decode_split_kernel(const __grid_constant__ CUtensorMap map, const DecodeArgs a) {
     constexpr int kStep = kWarps * kSub;  // warps of the split's CTAs
@@ -532,11 +533,12 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     // may be scheduled once every CTA of this grid has started; it still
     // waits for this grid to finish before reading.
     asm volatile("griddepcontrol.launch_dependents;");
-    if (kSub == 1 && kWarps == kWarpsNarrow && a.longest_first) {
+    if constexpr (kByLength) {
         // Row r of the grid is the r-th longest session (ties by batch row).
-        // Only the kernels of grids of several waves have this code: in the
-        // eight-warp one 48 layers of 12 sessions of 300 tokens took 167 us
-        // with it, never run, and 159 without.
+        // Kernels of their own: behind a test in the others, where it never
+        // ran, 48 layers of 12 sessions of 300 tokens took 167 us and 159
+        // without it, of 40 of 1 000 (fused) 779 and 773, and one call over 48
+        // layers of a session of 1K tokens 22.2 and 22.0.
         const int t = lane < a.B ? a.seq_lens[lane] : 0;
         int rank = 0;
         for (int j = 0; j < a.B; ++j) {
@@ -1175,9 +1177,9 @@ bool encode_hot_tensor_map(CUtensorMap *map, void *hot_base, int64_t rows, int64
     return true;
 }
 
-template <int kWarps, int kStages, int kSub>
+template <int kWarps, int kStages, int kSub, bool kByLength = false>
 static cudaError_t prepare_split() {
-    return cudaFuncSetAttribute(decode_split_kernel<kWarps, kStages, kSub>,
+    return cudaFuncSetAttribute(decode_split_kernel<kWarps, kStages, kSub, kByLength>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 decode_smem(kWarps, kStages));
 }
@@ -1190,6 +1192,8 @@ cudaError_t prepare_kernels() {
     if (e == cudaSuccess && set.maxDynamicSharedSizeBytes >= decode_smem(1, 8)) return e;
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1>();
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1>();
+    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1, true>();
+    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1, true>();
     if (e == cudaSuccess) e = prepare_split<8, 3, 1>();
     if (e == cudaSuccess) e = prepare_split<4, 6, 2>();
     if (e == cudaSuccess) e = prepare_split<4, 3, 2>();
@@ -1198,12 +1202,12 @@ cudaError_t prepare_kernels() {
     return e;
 }
 
-template <int kWarps, int kStages, int kSub>
+template <int kWarps, int kStages, int kSub, bool kByLength = false>
 static cudaError_t launch_split(cudaLaunchConfig_t &c, const CUtensorMap &map, const DecodeArgs &a) {
     c.gridDim.x *= kSub;
     c.blockDim = dim3(kWarps * 32);
     c.dynamicSmemBytes = decode_smem(kWarps, kStages);
-    return cudaLaunchKernelEx(&c, decode_split_kernel<kWarps, kStages, kSub>, map, a);
+    return cudaLaunchKernelEx(&c, decode_split_kernel<kWarps, kStages, kSub, kByLength>, map, a);
 }
 
 cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_sms,
@@ -1294,8 +1298,8 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     // 4K-60K 2 601 -> 2 531. Equal splits only lose by it, the block ids then
     // waiting for the ranks (24 of 1K-14K 2 879 and 2 920); a lane ranks one
     // session, so up to 32.
-    ka.longest_first = a.nlayers == 1 && a.B > 1 && a.B <= 32 && sub == 1 && ctas > 3 * sms &&
-                       split_tiles(a.max_blocks * a.s.bt) > KVT_SPLIT_MIN_TILES;
+    const bool by_length = a.nlayers == 1 && a.B > 1 && a.B <= 32 && sub == 1 && ctas > 3 * sms &&
+                           split_tiles(a.max_blocks * a.s.bt) > KVT_SPLIT_MIN_TILES;
     // Which sessions the split kernel merges itself (the bits are the same
     // either way): those of up to kSplitKernelMerge splits, in grids of at
     // least 8 CTAs per SM. There, many groups finish at different times and
@@ -1319,9 +1323,11 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     else if (ctas <= sms)
         e = launch_split<8, 3, 1>(c1, map, ka);
     else if (ctas <= 2 * sms || fill(2) > fill(3) + KVT_WAVE_MARGIN)
-        e = launch_split<kWarpsNarrow, kStagesHalf, 1>(c1, map, ka);
+        e = by_length ? launch_split<kWarpsNarrow, kStagesHalf, 1, true>(c1, map, ka)
+                      : launch_split<kWarpsNarrow, kStagesHalf, 1>(c1, map, ka);
     else
-        e = launch_split<kWarpsNarrow, kStagesFull, 1>(c1, map, ka);
+        e = by_length ? launch_split<kWarpsNarrow, kStagesFull, 1, true>(c1, map, ka)
+                      : launch_split<kWarpsNarrow, kStagesFull, 1>(c1, map, ka);
     if (e != cudaSuccess) return e;
     // Else the split kernel writes every session's output: one split each, or
     // few enough splits to merge there.

@@ -82,7 +82,6 @@ struct DecodeArgs {
     const uint16_t *k_new, *v_new;
     uint16_t *hot;            // pool base, written only when k_new is set
     int32_t pace;             // > 0: a warp's tiles in flight before the previous kernel ends
-    int32_t longest_first;    // 1: the grid's rows are the sessions by length
     int32_t inject_extra_tx;  // test hook: extra bytes expected on one tile (0 normally)
     Shape s;
 };
