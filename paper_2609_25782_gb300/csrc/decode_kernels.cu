@@ -971,6 +971,25 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     for (int h = warp; h < G; h += kWarps) merge_head_regs<kSplitKernelMerge / kMergeChains, true>(a, row_base + h, nsplit, lane);
 }
 
+// Splits of batch row b that a combine kernel has to merge; 0: none, its length
+// being bad or its splits merged by K1 (all sessions of one split, and of up to
+// `merged`; -1 where K1 leaves partials of every session, as shared splits do).
+// seq_lens is read before the combine's wait, as K1 reads it: no decode kernel
+// writes it, so only the partials have to wait for K1 to finish.
+// A row without splits to merge may leave at once, except in block 0: every
+// combine grid has a block that waits for K1, so that the end of the combine is
+// the end of the call. Where no row of a batch waited (sessions much shorter
+// than their table), the combine would end while K1's last CTAs still ran, and
+// what comes next, whose only predecessor is the combine (an overlapped call's
+// wait, a graph's next node), would start beside them: on the partials and
+// arrival counters that they still use, or before the outputs are written.
+__device__ __forceinline__ int splits_to_merge(const DecodeArgs &a, int b, int merged) {
+    const int T = a.seq_lens[b];
+    if (T < 1 || T > a.max_blocks * a.s.bt) return 0;
+    const int ns = num_splits(T);
+    return ns <= merged || (merged >= 0 && ns == 1) ? 0 : ns;
+}
+
 // K2 for tables of at most kRegMergeMax splits: one warp per (layer-batch
 // row, q-head), four per CTA, folding the four chains side by side from
 // registers (merge_head_regs), so no shared memory or CTA barrier sits
@@ -979,13 +998,10 @@ __global__ void __launch_bounds__(128) decode_combine_small_kernel(const DecodeA
     asm volatile("griddepcontrol.launch_dependents;");   // a following overlapped call
     const int64_t row = static_cast<int64_t>(blockIdx.x) * 4 + (threadIdx.x >> 5);
     if (row >= static_cast<int64_t>(a.nlayers) * a.B * a.s.Hq) return;
-    const int b = static_cast<int>((row / a.s.Hq) % a.B);
-    // seq_lens is read before the wait, as K1 reads it (no decode kernel writes it)
-    const int T = a.seq_lens[b];
-    if (T < 1 || T > a.max_blocks * a.s.bt) return;
-    const int ns = num_splits(T);
-    if (ns <= 1 || ns <= a.merge_max_splits) return;   // written by K1
+    const int ns = splits_to_merge(a, static_cast<int>((row / a.s.Hq) % a.B), a.merge_max_splits);
+    if (ns == 0 && blockIdx.x != 0) return;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (ns == 0) return;
     merge_head_regs<kRegMergeMax / kMergeChains, false>(a, row, ns, threadIdx.x & 31);
 }
 
@@ -1002,15 +1018,11 @@ template <int kParts, int kBatch>
 __global__ void __launch_bounds__(128) decode_combine_kernel(const DecodeArgs a) {
     asm volatile("griddepcontrol.launch_dependents;");   // a following overlapped call
     const int64_t row = blockIdx.x;                // lb * Hq + h
-    const int lb = static_cast<int>(row / a.s.Hq);
-    const int b = lb % a.B;
-    // seq_lens is read before the wait, as K1 reads it: no decode kernel
-    // writes it, so only the partials have to wait for K1 to finish.
-    const int T = a.seq_lens[b];
-    if (T < 1 || T > a.max_blocks * a.s.bt) return;
-    const int ns = num_splits(T);
-    if (kParts == 1 && (ns <= 1 || ns <= a.merge_max_splits)) return;   // written by K1
+    const int ns = splits_to_merge(a, static_cast<int>((row / a.s.Hq) % a.B),
+                                   kParts == 1 ? a.merge_max_splits : -1);
+    if (ns == 0 && blockIdx.x != 0) return;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (ns == 0) return;
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int64_t base = row * a.max_splits * kParts;
@@ -1076,10 +1088,8 @@ template <int kParts>
 __global__ void __launch_bounds__(128) decode_combine_shared_kernel(const DecodeArgs a) {
     asm volatile("griddepcontrol.launch_dependents;");   // a following overlapped call
     const int64_t row = blockIdx.x;                // lb * Hq + h
-    const int b = static_cast<int>((row / a.s.Hq) % a.B);
-    const int T = a.seq_lens[b];                   // before the wait, as K1 reads it
-    if (T < 1 || T > a.max_blocks * a.s.bt) return;
-    const int ns = num_splits(T);
+    const int ns = splits_to_merge(a, static_cast<int>((row / a.s.Hq) % a.B), -1);
+    if (ns == 0 && blockIdx.x != 0) return;
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const int s0 = (warp * ns) / kMergeChains;
@@ -1088,6 +1098,7 @@ __global__ void __launch_bounds__(128) decode_combine_shared_kernel(const Decode
     const float2 *ml = reinterpret_cast<const float2 *>(a.part_ml) + base;
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o + base * kHeadDim) + lane;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (ns == 0) return;
     __shared__ float s_m[kMergeChains], s_l[kMergeChains];
     __shared__ float4 s_acc[kMergeChains][kHeadDim / 4];
     constexpr int kPer = kRegMergeMax / kMergeChains;
