@@ -563,6 +563,9 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     const int T = a.seq_lens[b];
     if (T < 1 || T > a.max_blocks * sh.bt) {
         if (slice == 0 && g == 0 && threadIdx.x == 0) atomicOr(a.err, kErrBadLength);
+        // The end of a call of such rows alone is also the end of the call before:
+        // a third one waits for nothing else.
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }
     const int nsplit = num_splits(T);

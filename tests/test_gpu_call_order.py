@@ -76,3 +76,29 @@ def test_wide_tables(pkg, lens, tokens, bt):  # noqa: F811
         for got in (*outs, copies):
             assert torch.equal(got.double().cpu(), want)
     assert pool.check_device() == 0
+
+
+@pytest.mark.parametrize("n,tokens", [(1, 3000), (8, 4096), (24, 3000), (40, 700)])
+def test_call_of_bad_lengths_between_two_others(pkg, n, tokens):  # noqa: F811
+    """Rows of a bad length do no work, but a call of nothing else still ends after
+    the call before it: the next overlapped call waits for both."""
+    lens = [tokens - 7 * i for i in range(n)]
+    pool, _, tables, q = direct_case(pkg, lens, L=2, seed=43, max_batch=2 * n)
+    want = torch.from_numpy(np.concatenate([gpu_decode(pool, l, q, tables, lens) for l in range(2)]))
+    t = torch.as_tensor(tables, device="cuda")
+    s = torch.as_tensor(np.asarray(lens, dtype=np.int32), device="cuda")
+    bad = torch.zeros_like(s)
+    width, scale = t.shape[1], 1 / math.sqrt(128)
+    out, none = torch.empty(2, n, 32, 128, device="cuda"), torch.full((n, 32, 128), 7.0, device="cuda")
+    for _ in range(5):
+        out.fill_(float("nan"))
+        st = torch.cuda.current_stream()
+        pool.decode_attention(0, q[0], t, s, n, width, scale, out[0], st)
+        for _ in range(3):
+            pool.decode_attention(0, q[0], t, bad, n, width, scale, none, st, overlap_previous=True)
+        pool.decode_attention(1, q[1], t, s, n, width, scale, out[1], st, overlap_previous=True)
+        torch.cuda.synchronize()
+        assert torch.equal(out.double().cpu(), want)
+        assert torch.equal(none, torch.full_like(none, 7.0))
+        assert pool.check_device() == pkg.kvtier.KV_DEVICE_BAD_LENGTH
+    assert pool.check_device() == 0
