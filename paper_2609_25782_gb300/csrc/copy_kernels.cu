@@ -136,13 +136,13 @@ __device__ __forceinline__ void migrate_runs(const MigArgs &a, BlockOf block_of)
 // K3'/K4': block-granular moves for the residency mode: one warp per
 // (job, layer, K|V, kv-head) run; a job moves tokens [t0, t1) of one block.
 template <bool kPack>
-__global__ void __launch_bounds__(256) migrate_kernel(const MigArgs a) {
+__global__ void __launch_bounds__(kCopyThreads) migrate_kernel(const MigArgs a) {
     migrate_runs<kPack>(a, [&](int j) { return a.table[j]; });
 }
 
 // Resume-unpack with the new block ids in the launch parameters: the grid
 // also writes them to the session's table row (read by later work only).
-__global__ void __launch_bounds__(256) resume_inline_kernel(const __grid_constant__ ResumeArgs r) {
+__global__ void __launch_bounds__(kCopyThreads) resume_inline_kernel(const __grid_constant__ ResumeArgs r) {
     const int nthreads = gridDim.x * blockDim.x;
     int32_t *row = const_cast<int32_t *>(r.m.table);   // the pool's own row: writable
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < r.n; j += nthreads)
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(256) resume_inline_kernel(const __grid_constan
 }
 
 template <bool kPack>
-__global__ void __launch_bounds__(256) block_jobs_kernel(const __grid_constant__ BlockJobs a) {
+__global__ void __launch_bounds__(kCopyThreads) block_jobs_kernel(const __grid_constant__ BlockJobs a) {
     const Shape sh = a.s;
     const int runs = sh.L * 2 * sh.Hkv;
     const int cpb = sh.bt / kMigChunkTokens;      // chunks per block
@@ -246,7 +246,7 @@ __device__ __forceinline__ void append_tokens(const AppendArgs &a, BlockOf block
     }
 }
 
-__global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
+__global__ void __launch_bounds__(kCopyThreads) append_kernel(const AppendArgs a) {
     append_tokens(a, [&](int j) { return a.table[j]; });
 }
 
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) append_kernel(const AppendArgs a) {
 // to the session's table row (read by later work only), which saves the
 // table-write launch in front of it: a turn of 1 536 tokens, appended and
 // packed, 98.0 -> 94.3 us.
-__global__ void __launch_bounds__(256) append_inline_kernel(const __grid_constant__ AppendInlineArgs r) {
+__global__ void __launch_bounds__(kCopyThreads) append_inline_kernel(const __grid_constant__ AppendInlineArgs r) {
     const int nthreads = gridDim.x * blockDim.x;
     int32_t *row = const_cast<int32_t *>(r.m.table);   // the pool's own row: writable
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < r.n; j += nthreads)
@@ -285,16 +285,6 @@ __global__ void gather_tables_kernel(const __grid_constant__ GatherArgs a) {
 
 }  // namespace
 
-// One warp per item, 8 per CTA; at most `cap` CTAs (0: as many as a thread
-// index of 31 bits counts). The kernels stride over what is left.
-constexpr int64_t kMaxCtas = int64_t(1) << 23;
-static unsigned item_grid(int64_t items, int64_t cap) {
-    int64_t blocks = (items + 7) / 8;
-    if (cap <= 0 || cap > kMaxCtas) cap = kMaxCtas;
-    if (blocks > cap) blocks = cap;
-    return static_cast<unsigned>(blocks < 1 ? 1 : blocks);
-}
-
 // Chunks of a session's move, and whether it goes through the L2 once.
 static int64_t move_items(const MigArgs &a) {
     const int64_t nq = (a.t_end + kMigChunkTokens - 1) / kMigChunkTokens - a.t_begin / kMigChunkTokens;
@@ -307,21 +297,21 @@ static int32_t moves_once(int64_t items) {
 cudaError_t launch_unpack(MigArgs a, int max_ctas, cudaStream_t st) {
     if (a.t_end <= a.t_begin) return cudaSuccess;
     a.once = moves_once(move_items(a));
-    migrate_kernel<false><<<item_grid(move_items(a), max_ctas), 256, 0, st>>>(a);
+    migrate_kernel<false><<<item_grid(move_items(a), max_ctas), kCopyThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_unpack_inline(ResumeArgs &r, int max_ctas, cudaStream_t st) {
     if (r.m.t_end <= r.m.t_begin || r.n < 1 || r.n > kResumeInlineMax) return cudaErrorInvalidValue;
     r.m.once = moves_once(move_items(r.m));
-    resume_inline_kernel<<<item_grid(move_items(r.m), max_ctas), 256, 0, st>>>(r);
+    resume_inline_kernel<<<item_grid(move_items(r.m), max_ctas), kCopyThreads, 0, st>>>(r);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pack(MigArgs a, int max_ctas, cudaStream_t st) {
     if (a.t_end <= a.t_begin) return cudaSuccess;
     a.once = moves_once(move_items(a));
-    migrate_kernel<true><<<item_grid(move_items(a), max_ctas), 256, 0, st>>>(a);
+    migrate_kernel<true><<<item_grid(move_items(a), max_ctas), kCopyThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -331,13 +321,13 @@ static int64_t append_items(const AppendArgs &a) {
 }
 
 cudaError_t launch_append(const AppendArgs &a, cudaStream_t st) {
-    append_kernel<<<item_grid(append_items(a), 0), 256, 0, st>>>(a);
+    append_kernel<<<item_grid(append_items(a), 0), kCopyThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_append_inline(const AppendInlineArgs &r, cudaStream_t st) {
     if (r.n < 1 || r.n > kResumeInlineMax) return cudaErrorInvalidValue;
-    append_inline_kernel<<<item_grid(append_items(r.m), 0), 256, 0, st>>>(r);
+    append_inline_kernel<<<item_grid(append_items(r.m), 0), kCopyThreads, 0, st>>>(r);
     return cudaGetLastError();
 }
 
@@ -348,9 +338,9 @@ cudaError_t launch_block_jobs(BlockJobs &a, bool pack, int max_ctas, cudaStream_
     const unsigned grid = item_grid(items, max_ctas);
     a.once = moves_once(items);
     if (pack)
-        block_jobs_kernel<true><<<grid, 256, 0, st>>>(a);
+        block_jobs_kernel<true><<<grid, kCopyThreads, 0, st>>>(a);
     else
-        block_jobs_kernel<false><<<grid, 256, 0, st>>>(a);
+        block_jobs_kernel<false><<<grid, kCopyThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 

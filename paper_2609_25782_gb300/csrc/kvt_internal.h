@@ -125,6 +125,20 @@ struct AppendInlineArgs {
     int32_t blocks[kResumeInlineMax];
 };
 
+// Grid of a copy kernel: one warp per item, 8 per CTA; at most `cap` CTAs
+// (0: kMaxCtas). The kernels stride over what is left, with a grid's warps or,
+// over block ids, its threads as the stride, in int: the last index below the
+// end plus one stride has to fit.
+constexpr int kCopyThreads = 256;
+constexpr int64_t kMaxCtas = int64_t(1) << 22;
+static_assert(kMaxCtas * kCopyThreads + kResumeInlineMax <= INT32_MAX, "thread stride over block ids");
+inline unsigned item_grid(int64_t items, int64_t cap) {
+    int64_t blocks = (items + kCopyThreads / 32 - 1) / (kCopyThreads / 32);
+    if (cap <= 0 || cap > kMaxCtas) cap = kMaxCtas;
+    if (blocks > cap) blocks = cap;
+    return static_cast<unsigned>(blocks < 1 ? 1 : blocks);
+}
+
 // One block move between a hot slot and a session image: tokens [t0, t1) of
 // logical block j (all layers, K and V, all kv-heads).
 struct BlockJob {
