@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     const int st = split_tiles(T);
     const int tile0 = split * st;
     const int tile1 = min(tiles_of(T), tile0 + st);
-    const int my_tiles = (tile1 - tile0 - first + kStep - 1) / kStep;  // may be <= 0
+    int my_tiles = (tile1 - tile0 - first + kStep - 1) / kStep;  // may be <= 0
 
     uint8_t *ring = smem + warp * kStages * kTileBytes;
     const uint32_t ring_s = smem_u32(ring);
@@ -617,12 +617,25 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     };
     // The block of tile k, for every lane (k < 32 wherever it is used).
     auto blk_of = [&](int k) { return __shfl_sync(0xffffffffu, lane_blk, k & 31); };
+    // A wait ran out: tiles from .. to - 1 were issued and not consumed, so wait
+    // (again bounded) for them, that no copy lands after the CTA exits.
+    auto give_up = [&](int from, int to) {
+        if (lane == 0) atomicOr(a.err, kErrTimeout);
+#pragma unroll 1
+        for (int k = from; k < to; ++k) mbar_wait(bar0 + 8 * (k % kStages), (k / kStages) & 1);
+    };
     // a.pace > 0 (launch_decode): at most that many of the warp's tiles in
-    // flight while the previous kernel may still be running.
+    // flight while the previous kernel may still be running. A warp whose wait
+    // runs out here issues no more, and has no tiles to consume.
 #pragma unroll 1
     for (int k = 0; k < kStages && k < my_tiles; ++k) {
         const int blk = blk_of(k);
-        if (a.pace > 0 && k >= a.pace) mbar_wait(bar0 + 8 * (k - a.pace), 0);
+        if (a.pace > 0 && k >= a.pace &&
+            !__all_sync(0xffffffffu, mbar_wait(bar0 + 8 * (k - a.pace), 0))) {
+            give_up(k - a.pace, k);
+            my_tiles = 0;
+            break;
+        }
         if (lane == 0) issue(k, blk);
     }
 
@@ -905,14 +918,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         }
     }
 
-    if (fail_k >= 0) {
-        if (lane == 0) atomicOr(a.err, kErrTimeout);
-        // Tiles fail_k .. fail_k+kStages-1 were issued and not consumed: wait
-        // (again bounded) for them so no copy lands after the CTA exits.
-#pragma unroll 1
-        for (int k = fail_k; k < fail_k + kStages && k < my_tiles; ++k)
-            mbar_wait(bar0 + 8 * (k % kStages), (k / kStages) & 1);
-    }
+    if (fail_k >= 0) give_up(fail_k, min(fail_k + kStages, my_tiles));
 
     // Accumulator states -> this warp's own ring (all of its loads have
     // completed): accumulator v = warp + kWarps * i at float offset

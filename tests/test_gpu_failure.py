@@ -27,28 +27,40 @@ pytestmark = pytest.mark.gpu
 TOL = 1e-2
 
 
-def test_decode_wait_timeout_is_reported_and_context_survives(cuda_dev):
+# One warp's wait at its first tile (one 2 s limit), then the drain's re-wait of
+# that tile (another): in a two-session call of one split each (8 warps per CTA),
+# in splits shared by 8 CTAs, where tiles go in twos, and in the paced prologue
+# of an overlapped call, with splits shared by 2 CTAs (one and two per SM) and unshared.
+@pytest.mark.parametrize("lens,tokens,overlap", [
+    ([300, 77], 512, False), ([3000], 3008, False), ([16391], 16400, True),
+    ([4000] * 8, 4096, True), ([2100] * 20, 2112, True), ([3000], 3008, True)])
+def test_decode_wait_timeout_is_reported_and_context_survives(cuda_dev, lens, tokens, overlap):
     import __graft_entry__
     __graft_entry__.build()
     from paper_2609_25782_gb300 import Pool, kvtier
 
     L, Hq, Hkv, D, bt, seed = 1, 32, 4, 128, 16, 6
-    lens = [300, 77]
+    n = len(lens)
     nb = sum(-(-t // bt) for t in lens) + 4
-    pool = Pool(num_layers=L, num_hot_blocks=nb, cold_bytes=256, max_sessions=2, max_batch=2,
-                max_context=512)
+    pool = Pool(num_layers=L, num_hot_blocks=nb, cold_bytes=256, max_sessions=n, max_batch=n,
+                max_context=tokens)
     tables = synth.random_block_tables(seed, lens, bt, nb)
-    synth.fill_hot_pool_torch(pool.hot, seed, [0, 1], lens, tables, L, Hkv, D, bt)
-    q = synth.queries_torch(seed, [0, 1], range(L), Hq, D, cuda_dev)
+    synth.fill_hot_pool_torch(pool.hot, seed, range(n), lens, tables, L, Hkv, D, bt)
+    q = synth.queries_torch(seed, range(n), range(L), Hq, D, cuda_dev)
     t = torch.as_tensor(tables, device=cuda_dev)
     s = torch.as_tensor(np.asarray(lens, dtype=np.int32), device=cuda_dev)
-    hot = synth.hot_pool_np(seed, [0, 1], lens, tables, nb, L, Hkv, D, bt)
+    hot = synth.hot_pool_np(seed, range(n), lens, tables, nb, L, Hkv, D, bt)
     ref = oracle.paged_decode(hot, q.cpu().view(torch.int16).numpy().view(np.uint16), tables,
                               lens, 1 / math.sqrt(D), Hq)
 
-    def decode():
-        out = torch.full((L, 2, Hq, D), float("nan"), dtype=torch.float32, device=cuda_dev)
-        pool.decode_attention(0, q[0], t, s, 2, t.shape[1], 1 / math.sqrt(D), out[0])
+    def decode(arm=False):
+        out = torch.full((L, n, Hq, D), float("nan"), dtype=torch.float32, device=cuda_dev)
+        args = (0, q[0], t, s, n, t.shape[1], 1 / math.sqrt(D), out[0])
+        if overlap:
+            pool.decode_attention(*args)
+        if arm:
+            kvtier.kv_pool_inject_decode_timeout(pool.handle, 1)
+        pool.decode_attention(*args, overlap_previous=overlap)
         torch.cuda.synchronize()
         return out.double().cpu().numpy()
 
@@ -57,13 +69,12 @@ def test_decode_wait_timeout_is_reported_and_context_survives(cuda_dev):
 
     assert err(decode()) <= TOL and pool.check_device() == 0
 
-    kvtier.kv_pool_inject_decode_timeout(pool.handle, 1)
     t0 = time.monotonic()
-    decode()                                   # returns: the wait is bounded
+    decode(arm=True)                           # returns: the wait is bounded
     elapsed = time.monotonic() - t0
     flags = pool.check_device()
     assert flags == kvtier.KV_DEVICE_TIMEOUT
-    assert 1.5 < elapsed < 60                  # one 2 s limit (plus the bounded drain)
+    assert 1.5 < elapsed < 5                   # the wait and the drain's, 2 s each
     assert "timed out" in kvtier.kv_last_error() or "flags 4" in kvtier.kv_last_error()
 
     # the hook disarmed itself and the context is intact
