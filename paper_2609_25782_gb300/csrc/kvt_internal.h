@@ -111,8 +111,9 @@ struct AppendArgs {
     const uint8_t *k, *v;     // [L][n][Hkv][D] bf16
     const int32_t *table;
     uint8_t *hot;
-    int64_t pos0;
+    int32_t pos0;             // contexts hold at most 2^30 tokens
     int32_t n;
+    int32_t group, groups, head_inv;   // set by the launch: tokens per item, items per layer
     int32_t *err;
     Shape s;
 };
@@ -196,8 +197,8 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
 cudaError_t launch_unpack(MigArgs a, int max_ctas, cudaStream_t st);
 cudaError_t launch_unpack_inline(ResumeArgs &r, int max_ctas, cudaStream_t st);
 cudaError_t launch_pack(MigArgs a, int max_ctas, cudaStream_t st);
-cudaError_t launch_append(const AppendArgs &a, cudaStream_t st);
-cudaError_t launch_append_inline(const AppendInlineArgs &r, cudaStream_t st);
+cudaError_t launch_append(AppendArgs a, cudaStream_t st);
+cudaError_t launch_append_inline(AppendInlineArgs &r, cudaStream_t st);
 cudaError_t launch_block_jobs(BlockJobs &a, bool pack, int max_ctas, cudaStream_t st);
 cudaError_t launch_table_write(const TableWriteArgs &a, cudaStream_t st);
 cudaError_t launch_gather(const GatherArgs &a, cudaStream_t st);

@@ -238,7 +238,7 @@ struct kv_pool {
         a.v = static_cast<const uint8_t *>(v);
         a.table = d_tables + static_cast<int64_t>(sid) * table_stride;
         a.hot = static_cast<uint8_t *>(cfg.hot_base);
-        a.pos0 = s.T;
+        a.pos0 = static_cast<int32_t>(s.T);
         a.n = n;
         a.err = d_err;
         a.s = shape;
