@@ -400,8 +400,9 @@ int kv_pool_check_device(kv_pool *pool, int32_t *flags);
 /* Cap the migration kernels (resume-unpack, pause-pack, evictions) at
  * max_ctas CTAs of 256 threads, so that migrations running beside decode take
  * a smaller share of HBM bandwidth (Section 3, data paths: eviction and resume
- * overlap decode). 0 removes the cap (the default: a warp per 8-token chunk of
- * each layer's K and V runs).
+ * overlap decode). 0 removes the cap (the default): then a warp takes one 8-token
+ * chunk of each layer's K and V runs, or, on another stream than the pool's last
+ * decode call, where decode may run beside the move, 16 CTAs per SM share them.
  * Affects later calls only. */
 int kv_pool_set_migration_limit(kv_pool *pool, int32_t max_ctas);
 

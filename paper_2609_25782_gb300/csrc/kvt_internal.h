@@ -140,6 +140,23 @@ inline unsigned item_grid(int64_t items, int64_t cap) {
     return static_cast<unsigned>(blocks < 1 ? 1 : blocks);
 }
 
+// CTAs of a migration, 0 for a warp per item; limit: the caller's bound, 0 for
+// none. A grid of a warp per item hands its SM slots, CTA by CTA, to the decode
+// calls of a stream that comes first, so where decode may run beside the move
+// its CTAs are few and stride over the items. An agentic trace of 16 decoding
+// sessions, decode on a high-priority stream: a resume took 3.9 ms (p50; p99
+// 15.5) with a warp per item, 1.85 (5.4) with 32 CTAs per SM, 1.2 (2.7) with
+// 16, 0.97 (1.9) with 8 and 0.76 (2.0) with 6, the decode steps 3.83 ms in all of
+// them. By itself the move is the faster the more CTAs it has: three sessions
+// of 12K-32K tokens resumed twice 4.38 ms, 4.56, 4.64, 4.73 and 4.89. 16 keep
+// what 16-byte loads and 32 CTAs per SM reached (2.05 ms and 4.61).
+constexpr int kBesideCtasPerSm = 16;
+inline int migration_ctas(int limit, bool beside_decode, int num_sms) {
+    const int most = beside_decode ? kBesideCtasPerSm * num_sms : 0;
+    if (limit <= 0 || (most > 0 && most < limit)) return most;
+    return limit;
+}
+
 // One block move between a hot slot and a session image: tokens [t0, t1) of
 // logical block j (all layers, K and V, all kv-heads).
 struct BlockJob {
@@ -193,7 +210,7 @@ cudaError_t prepare_kernels();  // per-device function attributes
 // split kernel's tile rings to the grid.
 cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_sms,
                           cudaStream_t st, bool overlap_previous);
-// max_ctas > 0 caps the migration grids (kv_pool_set_migration_limit).
+// max_ctas > 0 caps the migration grids (migration_ctas).
 cudaError_t launch_unpack(MigArgs a, int max_ctas, cudaStream_t st);
 cudaError_t launch_unpack_inline(ResumeArgs &r, int max_ctas, cudaStream_t st);
 cudaError_t launch_pack(MigArgs a, int max_ctas, cudaStream_t st);

@@ -108,6 +108,10 @@ struct kv_pool {
     int64_t part_alloc = 0;              // partial rows allocated (at least part_rows)
     int num_sms = 1;
     int mig_ctas = 0;                    // cap on migration-kernel CTAs, 0 = none
+    // Stream of the last decode call: moves on another one may run beside
+    // decode. Compared only, and only to size a grid.
+    bool decoded = false;
+    cudaStream_t decode_stream = nullptr;
     kvt::Shape shape{};
 
     std::vector<int32_t> free_list;      // top = back
@@ -151,6 +155,10 @@ struct kv_pool {
         if (e != cudaSuccess)
             return fail(KV_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
         return KV_OK;
+    }
+
+    int move_ctas(cudaStream_t st) const {
+        return kvt::migration_ctas(mig_ctas, decoded && st != decode_stream, num_sms);
     }
 
     Session *session(int32_t sid) {
@@ -392,7 +400,7 @@ struct kv_pool {
             a.once = 0;
             std::copy(jobs.begin() + i, jobs.begin() + i + a.n, a.job);
             int rc = cuda(pack ? "pack launch" : "unpack launch",
-                          [&] { return kvt::launch_block_jobs(a, pack, mig_ctas, st); });
+                          [&] { return kvt::launch_block_jobs(a, pack, move_ctas(st), st); });
             if (rc) return rc;
         }
         return KV_OK;
@@ -936,6 +944,8 @@ static int decode_impl(kv_pool *p, int32_t layer, const void *q, const void *k_n
     int rc = p->cuda("decode launch", [&] { return kvt::launch_decode(p->tmap, a, p->num_sms, st, overlap); });
     if (rc) return rc;
     p->inject_timeout = false;
+    p->decoded = true;
+    p->decode_stream = st;
     p->stats.decodes += 1;
     return KV_OK;
 }
@@ -986,7 +996,7 @@ int session_pause(kv_pool *p, int32_t sid, kv_stream_t stream_) {
         kvt::MigArgs m = p->mig_args(sid, *s);
         m.t_begin = static_cast<int32_t>(t0);
         m.t_end = static_cast<int32_t>(t1);
-        rc = p->cuda("pack launch", [&] { return kvt::launch_pack(m, p->mig_ctas, st); });
+        rc = p->cuda("pack launch", [&] { return kvt::launch_pack(m, p->move_ctas(st), st); });
     }
     if (!rc) rc = p->cuda("cudaEventRecord", [&] { return cudaEventRecord(p->fences[f].ev, st); });
     if (rc) return rc;
@@ -1048,7 +1058,7 @@ int session_resume(kv_pool *p, int32_t sid, kv_stream_t stream_) {
         r.pad = 0;
         std::memcpy(r.blocks, fresh.data(), sizeof(int32_t) * need);
         rc = p->cuda("unpack launch",
-                     [&] { return kvt::launch_unpack_inline(r, p->mig_ctas, st); });
+                     [&] { return kvt::launch_unpack_inline(r, p->move_ctas(st), st); });
     } else if (!rc) {
         rc = p->write_table(sid, fresh.data(), 0, need, st);
         if (!rc) {
@@ -1056,7 +1066,7 @@ int session_resume(kv_pool *p, int32_t sid, kv_stream_t stream_) {
             m.t_begin = 0;
             m.t_end = static_cast<int32_t>(s->T);
             rc = p->cuda("unpack launch",
-                         [&] { return kvt::launch_unpack(m, p->mig_ctas, st); });
+                         [&] { return kvt::launch_unpack(m, p->move_ctas(st), st); });
         }
     }
     if (!rc) rc = p->cuda("cudaEventRecord", [&] { return cudaEventRecord(s->ready, st); });

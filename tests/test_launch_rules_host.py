@@ -17,3 +17,14 @@ def test_copy_grid_strides_in_int(items, cap):
     most = 2 ** 31 - 1
     assert r.inline_blocks() - 1 + ctas * threads <= most
     assert min(items, 1 << 28) - 1 + ctas * threads // 32 <= most
+
+
+@pytest.mark.parametrize("sms", [132, 152])
+def test_migrations_beside_decode_stride(sms):
+    """A move that decode may run beside is a few CTAs an SM, which keep their slots; one by
+    itself has no bound; the caller's limit holds in both."""
+    ctas = rules().migration_ctas
+    assert ctas(0, 0, sms) == 0 and ctas(0, 1, sms) == 16 * sms
+    for limit in (1, 8, sms, 16 * sms - 1):
+        assert ctas(limit, 0, sms) == ctas(limit, 1, sms) == limit
+    assert ctas(1 << 20, 0, sms) == 1 << 20 and ctas(1 << 20, 1, sms) == 16 * sms
