@@ -55,9 +55,10 @@ constexpr int kHalfBytes = 2048;           // 16 rows x 128 B (64 dims)
 //                                   and w + 4 and alternates between them, so
 //                                   consecutive tiles of a warp are independent
 //   <4 warps, 3 slots, 1>           2 CTAs per SM
-//   the same two, true              their CTAs take the longest sessions first
 //   <8 warps, 3 slots, 1>           1 CTA per SM: one accumulator per warp,
 //                                   twice the warps per SM
+//   the first two, kLongestFirst    their CTAs take the longest sessions first
+//   these three, kOneSplit          tables of one split (kernel forms, below)
 //   <8 / kSub warps, slots, kSub>   a split shared by kSub = 2 or 8 CTAs, one
 //                                   accumulator per warp: grids of up to
 //                                   three CTAs per SM once shared
@@ -74,7 +75,6 @@ constexpr int kStagesHalf = 3;             // 2 CTAs per SM
 __host__ __device__ constexpr int decode_smem(int warps, int stages) {
     return warps * stages * kTileBytes + 1024 + 256;   // rings, alignment, barriers
 }
-static_assert(kWarpsNarrow * kStagesHalf * 8 <= 256, "mbarriers must fit their 256-byte area");
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -138,8 +138,10 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 // the default policy and this one, 16 x 14K tokens 72.7 and 70.2, 32 x 20K 191
 // and 185.5, 64 x 8K 154.3 and 150.4, 8 x 16K 45.2 and 44.1, 256 x 4K (merged
 // in the split kernel) 309 and 302; sessions whose layer fits the L2 the same.
-// Sessions of one split leave no partials and keep the default (256 x 1 000
-// 80.3 and 81.2).
+// Sessions of one split leave no partials and keep the normal policy (256 x 1 000
+// 80.3 and 81.2 with evict-first); tables of one split name none at all: with
+// K and V in the L2 a call over 48 layers of one session of 1K tokens takes 18.4 us
+// with the normal policy spelled out and 16.5 without.
 __device__ __forceinline__ uint64_t copy_policy(bool stream) {
     uint64_t p, q;
     asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
@@ -149,8 +151,17 @@ __device__ __forceinline__ uint64_t copy_policy(bool stream) {
 
 // One tile: the box (64 columns, 16 rows, 2 column halves, K and V) of the
 // hot pool's 4-D view, starting at K row `row`.
+template <bool kPolicy>
 __device__ __forceinline__ void tma_load_tile(uint32_t dst, const CUtensorMap *map, int row,
                                               uint32_t bar, uint64_t policy) {
+    if constexpr (!kPolicy) {
+        asm volatile(
+            "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+            " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(dst),
+            "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(0), "r"(0), "r"(bar)
+            : "memory");
+        return;
+    }
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
         ".L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(dst),
@@ -428,7 +439,7 @@ constexpr int kAccFloats = kMaxGroup * kOStride + 2 * kMaxGroup;   // O rows, m[
 // head, four dims per lane, so a warp reads one head's row of a state as 32
 // consecutive float4. A session of one split held by one CTA is finished here;
 // others leave partials.
-template <int kHere, int kSub, int kWarps, typename State>
+template <int kHere, int kSub, int kWarps, bool kOne, typename State>
 __device__ __forceinline__ void merge_states(const DecodeArgs &a, int64_t row_base, int G,
                                              int nsplit, int split, int sub, State state) {
     constexpr int kParts = parts_per_split(kSub);   // of the split
@@ -447,7 +458,7 @@ __device__ __forceinline__ void merge_states(const DecodeArgs &a, int64_t row_ba
             acc[v] = *reinterpret_cast<const float4 *>(ws + h * kOStride + d0);
         }
         if constexpr (kMine == 1) join_accs<kHere>(m, l, acc);
-        if (kSub == 1 && nsplit == 1) {
+        if (kOne || (kSub == 1 && nsplit == 1)) {
             const float inv = __frcp_rn(l[0]);
             store_out(a, row_base + h, lane,
                       make_float4(__fmul_rn(acc[0].x, inv), __fmul_rn(acc[0].y, inv),
@@ -497,11 +508,26 @@ struct AccState {
     float o[8][4];  // O^T fragments
 };
 
-template <int kWarps, int kStages, int kSub, bool kByLength = false>
+// Forms of the kernel, each of its own so that the others do not carry its code:
+// kLongestFirst takes the sessions by length (launch_decode); kOneSplit is for
+// tables of one split, whose calls are a chain of latencies: no L2 policy, no
+// pacing, no partials or arrival, and a ring that is filled without a loop and
+// refilled without a branch around the block id's shuffle. us in the form for any
+// table and in this one: 48 layers one after another, one session of 1K tokens
+// 303.5 and 290.1, of 300 151.4 and 149.1, 8 of 1K 327.5 and 320.3, 40 of 1 000 741
+// and 726, 128 of 1 000 2 000 and 1 983, but 12 of 300 174.3 and 180.4; all
+// layers in one call, one session of 1K 18.2 and 16.5 with K and V in the L2, 21.5
+// and 21.0 from HBM, 12 of 300 67.4 and 64.2.
+enum Form { kAny, kLongestFirst, kOneSplit };
+
+template <int kWarps, int kStages, int kSub, Form kForm = kAny>
 __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kStages == 2 ? 3 : kStages == 3 ? 2 : 1)
     decode_split_kernel(const __grid_constant__ CUtensorMap map, const DecodeArgs a) {
     constexpr int kStep = kWarps * kSub;  // warps of the split's CTAs
     constexpr int kA = kAccs / kStep;     // accumulators per warp
+    static_assert(kWarps * kStages * 8 <= 256, "mbarriers must fit their 256-byte area");
+    constexpr bool kOne = kForm == kOneSplit;
+    static_assert(!kOne || kSub == 1, "one split: unshared");
     static_assert(kA * kStep == kAccs, "accumulators divide among the warps");
     static_assert(kA == 1 || (kA == 2 && kSub == 1), "two accumulators only in an unshared split");
     extern __shared__ uint8_t smem_raw[];
@@ -533,12 +559,11 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     // may be scheduled once every CTA of this grid has started; it still
     // waits for this grid to finish before reading.
     asm volatile("griddepcontrol.launch_dependents;");
-    if constexpr (kByLength) {
+    if constexpr (kForm == kLongestFirst) {
         // Row r of the grid is the r-th longest session (ties by batch row).
-        // Kernels of their own: behind a test in the others, where it never
-        // ran, 48 layers of 12 sessions of 300 tokens took 167 us and 159
-        // without it, of 40 of 1 000 (fused) 779 and 773, and one call over 48
-        // layers of a session of 1K tokens 22.2 and 22.0.
+        // Behind a test in the other forms, where it never ran, 48 layers of 12
+        // sessions of 300 tokens took 167 us and 159 without it, of 40 of 1 000
+        // (fused) 779 and 773.
         const int t = lane < a.B ? a.seq_lens[lane] : 0;
         int rank = 0;
         for (int j = 0; j < a.B; ++j) {
@@ -554,7 +579,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     // Lanes past the session's tiles may read table entries past its blocks
     // (never used).
     constexpr int kMinWarpTiles = KVT_SPLIT_MIN_TILES / kStep;
-    const bool fixed_split = split_tiles(a.max_blocks * sh.bt) == KVT_SPLIT_MIN_TILES;
+    const bool fixed_split = kOne || split_tiles(a.max_blocks * sh.bt) == KVT_SPLIT_MIN_TILES;
     int early_blk = 0;
     if (fixed_split && lane < kMinWarpTiles) {
         const int j = (split * KVT_SPLIT_MIN_TILES + first + lane * kStep) * kTileTokens / sh.bt;
@@ -568,11 +593,11 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }
-    const int nsplit = num_splits(T);
+    const int nsplit = kOne ? 1 : num_splits(T);
     if (split >= nsplit) return;
     const int st = split_tiles(T);
-    const int tile0 = split * st;
-    const int tile1 = min(tiles_of(T), tile0 + st);
+    const int tile0 = kOne ? 0 : split * st;
+    const int tile1 = kOne ? tiles_of(T) : min(tiles_of(T), tile0 + st);
     int my_tiles = (tile1 - tile0 - first + kStep - 1) / kStep;  // may be <= 0
 
     uint8_t *ring = smem + warp * kStages * kTileBytes;
@@ -613,7 +638,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         // one barrier then never completes its phase, although every copy lands.
         const bool injected = k == 0 && warp == 0 && slice == 0 && g == 0 && lb == 0;
         mbar_expect_tx(bar, kTileBytes + (injected ? a.inject_extra_tx : 0));
-        tma_load_tile(slot, &map, rowk, bar, policy);
+        tma_load_tile<!kOne>(slot, &map, rowk, bar, policy);
     };
     // The block of tile k, for every lane (k < 32 wherever it is used).
     auto blk_of = [&](int k) { return __shfl_sync(0xffffffffu, lane_blk, k & 31); };
@@ -627,6 +652,13 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     // a.pace > 0 (launch_decode): at most that many of the warp's tiles in
     // flight while the previous kernel may still be running. A warp whose wait
     // runs out here issues no more, and has no tiles to consume.
+    if constexpr (kOne) {
+#pragma unroll
+        for (int k = 0; k < kStages; ++k) {
+            const int blk = blk_of(k);
+            if (lane == 0 && k < my_tiles) issue(k, blk);
+        }
+    } else {
 #pragma unroll 1
     for (int k = 0; k < kStages && k < my_tiles; ++k) {
         const int blk = blk_of(k);
@@ -637,6 +669,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
             break;
         }
         if (lane == 0) issue(k, blk);
+    }
     }
 
     uint32_t koff[4], voff[4];
@@ -746,9 +779,9 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     };
     auto slot_of = [&](int k) { return ring_s + (k % kStages) * kTileBytes; };
     auto refill = [&](int k) {
-        if (k + kStages >= my_tiles) return;
+        if (!kOne && k + kStages >= my_tiles) return;
         const int nblk = blk_of(k + kStages);
-        if (lane == 0) issue(k + kStages, nblk);
+        if (lane == 0 && k + kStages < my_tiles) issue(k + kStages, nblk);
     };
 
     // One tile into accumulator s. False: its wait timed out.
@@ -954,12 +987,12 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     __syncthreads();
 
     const int64_t row_base = static_cast<int64_t>(lb) * sh.Hq + g * G;
-    merge_states<kAccs / kSub, kSub, kWarps>(
+    merge_states<kAccs / kSub, kSub, kWarps, kOne>(
         a, row_base, G, nsplit, split, sub, [&](int v) {
             return reinterpret_cast<const float *>(smem + (v % kWarps) * kStages * kTileBytes) +
                    (v / kWarps) * kAccFloats;
         });
-    if (kWarps != kWarpsNarrow || kSub > 1) return;
+    if (kOne || kWarps != kWarpsNarrow || kSub > 1) return;
     if (nsplit == 1 || nsplit > a.merge_max_splits) return;
 
     // Arrival. Every split of the group arrives once, whatever happened in
@@ -1197,9 +1230,9 @@ bool encode_hot_tensor_map(CUtensorMap *map, void *hot_base, int64_t rows, int64
     return true;
 }
 
-template <int kWarps, int kStages, int kSub, bool kByLength = false>
+template <int kWarps, int kStages, int kSub, Form kForm = kAny>
 static cudaError_t prepare_split() {
-    return cudaFuncSetAttribute(decode_split_kernel<kWarps, kStages, kSub, kByLength>,
+    return cudaFuncSetAttribute(decode_split_kernel<kWarps, kStages, kSub, kForm>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 decode_smem(kWarps, kStages));
 }
@@ -1212,9 +1245,12 @@ cudaError_t prepare_kernels() {
     if (e == cudaSuccess && set.maxDynamicSharedSizeBytes >= decode_smem(1, 8)) return e;
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1>();
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1>();
-    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1, true>();
-    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1, true>();
+    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1, kLongestFirst>();
+    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1, kLongestFirst>();
     if (e == cudaSuccess) e = prepare_split<8, 3, 1>();
+    if (e == cudaSuccess) e = prepare_split<8, 3, 1, kOneSplit>();
+    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1, kOneSplit>();
+    if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1, kOneSplit>();
     if (e == cudaSuccess) e = prepare_split<4, 6, 2>();
     if (e == cudaSuccess) e = prepare_split<4, 3, 2>();
     if (e == cudaSuccess) e = prepare_split<4, 2, 2>();
@@ -1222,12 +1258,12 @@ cudaError_t prepare_kernels() {
     return e;
 }
 
-template <int kWarps, int kStages, int kSub, bool kByLength = false>
+template <int kWarps, int kStages, int kSub, Form kForm = kAny>
 static cudaError_t launch_split(cudaLaunchConfig_t &c, const CUtensorMap &map, const DecodeArgs &a) {
     c.gridDim.x *= kSub;
     c.blockDim = dim3(kWarps * 32);
     c.dynamicSmemBytes = decode_smem(kWarps, kStages);
-    return cudaLaunchKernelEx(&c, decode_split_kernel<kWarps, kStages, kSub, kByLength>, map, a);
+    return cudaLaunchKernelEx(&c, decode_split_kernel<kWarps, kStages, kSub, kForm>, map, a);
 }
 
 cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_sms,
@@ -1340,13 +1376,19 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
         e = launch_split<4, 3, 2>(c1, map, ka);
     else if (sub == 2)
         e = launch_split<4, 2, 2>(c1, map, ka);
+    else if (splits == 1 && ctas <= sms)
+        e = launch_split<8, 3, 1, kOneSplit>(c1, map, ka);
+    else if (splits == 1)
+        e = ctas <= 2 * sms || fill(2) > fill(3) + KVT_WAVE_MARGIN
+                ? launch_split<kWarpsNarrow, kStagesHalf, 1, kOneSplit>(c1, map, ka)
+                : launch_split<kWarpsNarrow, kStagesFull, 1, kOneSplit>(c1, map, ka);
     else if (ctas <= sms)
         e = launch_split<8, 3, 1>(c1, map, ka);
     else if (ctas <= 2 * sms || fill(2) > fill(3) + KVT_WAVE_MARGIN)
-        e = by_length ? launch_split<kWarpsNarrow, kStagesHalf, 1, true>(c1, map, ka)
+        e = by_length ? launch_split<kWarpsNarrow, kStagesHalf, 1, kLongestFirst>(c1, map, ka)
                       : launch_split<kWarpsNarrow, kStagesHalf, 1>(c1, map, ka);
     else
-        e = by_length ? launch_split<kWarpsNarrow, kStagesFull, 1, true>(c1, map, ka)
+        e = by_length ? launch_split<kWarpsNarrow, kStagesFull, 1, kLongestFirst>(c1, map, ka)
                       : launch_split<kWarpsNarrow, kStagesFull, 1>(c1, map, ka);
     if (e != cudaSuccess) return e;
     // Else the split kernel writes every session's output: one split each, or

@@ -80,3 +80,29 @@ def test_longest_first(pkg, n, bt):  # noqa: F811
                               1 / math.sqrt(128), 32)
     assert scaled_err(got, ref[0]) <= TOL
     assert pool.check_device() == 0
+
+
+# Tables of one split run kernels of their own, at 1, 2 and 3 CTAs per SM: the bits are those of
+# the same sessions in tables of two splits.
+@pytest.mark.parametrize("n", [9, 45, 99])
+@pytest.mark.parametrize("bt,hkv", [(16, 4), (64, 4), (16, 1)])
+def test_tables_of_one_split(pkg, n, bt, hkv):  # noqa: F811
+    lens = ([1, 15, 16, 17, 127, 128, 129, 1023, 1024] * 11)[:n]
+    pool, sess, tables, q = direct_case(pkg, lens, L=2, Hq=8 * hkv, Hkv=hkv, bt=bt, seed=19,
+                                        max_batch=4 * n)
+    pool._scale = 0.5
+    wide = np.pad(tables, ((0, 0), (0, tables.shape[1])), constant_values=-1)
+    got = gpu_decode(pool, -1, q, tables, lens)
+    assert np.array_equal(got.view(np.int64), gpu_decode(pool, -1, q, wide, lens).view(np.int64))
+    ref = oracle.paged_decode(host_hot(pool, 19, sess, lens, tables),
+                              q.cpu().view(torch.int16).numpy().view(np.uint16), tables, lens, 0.5,
+                              8 * hkv)
+    assert scaled_err(got, ref) <= TOL
+    t = torch.as_tensor(tables, device="cuda")
+    s = torch.as_tensor(np.asarray(lens, dtype=np.int32), device="cuda")
+    out = torch.empty(2, n, 8 * hkv, 128, device="cuda")
+    for l in range(2):
+        pool.decode_attention(l, q[l].contiguous(), t, s, n, t.shape[1], 0.5, out[l], overlap_previous=l > 0)
+    torch.cuda.synchronize()
+    assert np.array_equal(out.double().cpu().numpy().view(np.int64), got.view(np.int64))
+    assert pool.check_device() == 0
