@@ -338,16 +338,16 @@ static int64_t append_shape(AppendArgs &a) {
     return static_cast<int64_t>(a.s.L) * a.groups;
 }
 
-cudaError_t launch_append(AppendArgs a, cudaStream_t st) {
+cudaError_t launch_append(AppendArgs a, int max_ctas, cudaStream_t st) {
     const int64_t items = append_shape(a);
-    append_kernel<<<item_grid(items, 0), kCopyThreads, 0, st>>>(a);
+    append_kernel<<<item_grid(items, max_ctas), kCopyThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_append_inline(AppendInlineArgs &r, cudaStream_t st) {
+cudaError_t launch_append_inline(AppendInlineArgs &r, int max_ctas, cudaStream_t st) {
     if (r.n < 1 || r.n > kResumeInlineMax) return cudaErrorInvalidValue;
     const int64_t items = append_shape(r.m);
-    append_inline_kernel<<<item_grid(items, 0), kCopyThreads, 0, st>>>(r);
+    append_inline_kernel<<<item_grid(items, max_ctas), kCopyThreads, 0, st>>>(r);
     return cudaGetLastError();
 }
 

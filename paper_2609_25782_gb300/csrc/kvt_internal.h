@@ -210,12 +210,12 @@ cudaError_t prepare_kernels();  // per-device function attributes
 // split kernel's tile rings to the grid.
 cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_sms,
                           cudaStream_t st, bool overlap_previous);
-// max_ctas > 0 caps the migration grids (migration_ctas).
+// max_ctas > 0 caps the copy grids (migration_ctas).
 cudaError_t launch_unpack(MigArgs a, int max_ctas, cudaStream_t st);
 cudaError_t launch_unpack_inline(ResumeArgs &r, int max_ctas, cudaStream_t st);
 cudaError_t launch_pack(MigArgs a, int max_ctas, cudaStream_t st);
-cudaError_t launch_append(AppendArgs a, cudaStream_t st);
-cudaError_t launch_append_inline(AppendInlineArgs &r, cudaStream_t st);
+cudaError_t launch_append(AppendArgs a, int max_ctas, cudaStream_t st);
+cudaError_t launch_append_inline(AppendInlineArgs &r, int max_ctas, cudaStream_t st);
 cudaError_t launch_block_jobs(BlockJobs &a, bool pack, int max_ctas, cudaStream_t st);
 cudaError_t launch_table_write(const TableWriteArgs &a, cudaStream_t st);
 cudaError_t launch_gather(const GatherArgs &a, cudaStream_t st);

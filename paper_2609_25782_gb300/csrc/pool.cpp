@@ -157,8 +157,9 @@ struct kv_pool {
         return KV_OK;
     }
 
+    bool beside_decode(cudaStream_t st) const { return decoded && st != decode_stream; }
     int move_ctas(cudaStream_t st) const {
-        return kvt::migration_ctas(mig_ctas, decoded && st != decode_stream, num_sms);
+        return kvt::migration_ctas(mig_ctas, beside_decode(st), num_sms);
     }
 
     Session *session(int32_t sid) {
@@ -250,14 +251,16 @@ struct kv_pool {
         a.n = n;
         a.err = d_err;
         a.s = shape;
+        // the caller's bound is for migrations alone
+        const int ctas = kvt::migration_ctas(0, beside_decode(st), num_sms);
         if (fresh_n > 0 && fresh_n <= kvt::kResumeInlineMax) {
             r.from = static_cast<int32_t>(from);
             r.n = static_cast<int32_t>(fresh_n);
             std::memcpy(r.blocks, vals, sizeof(int32_t) * fresh_n);
-            return cuda("append launch", [&] { return kvt::launch_append_inline(r, st); });
+            return cuda("append launch", [&] { return kvt::launch_append_inline(r, ctas, st); });
         }
         int rc = fresh_n > 0 ? write_table(sid, vals, from, fresh_n, st) : KV_OK;
-        if (!rc) rc = cuda("append launch", [&] { return kvt::launch_append(a, st); });
+        if (!rc) rc = cuda("append launch", [&] { return kvt::launch_append(a, ctas, st); });
         return rc;
     }
 

@@ -41,11 +41,12 @@ def test_pack_and_unpack_at_chunk_edges(cuda_dev, bt, lru, t1, t2):
 @pytest.mark.parametrize("lru", [False, True])
 def test_moves_on_another_stream_than_decode(cuda_dev, lru):
     """After a decode call, moves on another stream take the grid whose CTAs stride over the
-    chunks: 64 runs of 501 chunks are more than the 8 warps of 16 CTAs on each SM."""
+    chunks: 64 runs of 901 chunks are more than the 8 warps of 16 CTAs on each SM, and so
+    are 8 layers of 3 601 groups of two tokens."""
     import __graft_entry__
     __graft_entry__.build()
     from paper_2609_25782_gb300 import Pool
-    L, hkv, d, t, bt = 8, 4, 128, 4001, 16
+    L, hkv, d, t, bt = 8, 4, 128, 7201, 16
     nb = -(-t // bt)
     pool = Pool(num_layers=L, num_hot_blocks=nb, cold_bytes=2 * nb * bt * L * 2 * hkv * d * 2,
                 num_q_heads=hkv, num_kv_heads=hkv, max_sessions=2, max_batch=1, max_context=t,
@@ -65,8 +66,12 @@ def test_moves_on_another_stream_than_decode(cuda_dev, lru):
     side.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(side):
         pool.session_pause(sid, side)
-        pool.session_append(other, torch.zeros_like(kv[0]), torch.zeros_like(kv[1]), side)
+        # appended there too
+        pool.session_append(other, kv[1], kv[0], side)
         assert torch.equal(pool.image(sid), want)
+        row = torch.as_tensor(pool.session_block_table(other), device="cuda", dtype=torch.int64)
+        got = pool.hot_view()[row].permute(1, 2, 3, 0, 4, 5).reshape(L, 2, hkv, -1, d)
+        assert torch.equal(got[:, :, :, :t], want.flip(1))
         pool.session_destroy(other)
         pool.shuffle_free(3)
         pool.session_resume(sid, side)
