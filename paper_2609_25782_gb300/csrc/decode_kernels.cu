@@ -511,9 +511,8 @@ struct AccState {
 // Forms of the kernel, each of its own so that the others do not carry its code:
 // kLongestFirst takes the sessions by length (launch_decode); kOneSplit is for
 // tables of one split, whose calls are a chain of latencies: no L2 policy, no
-// pacing, no partials or arrival, and a ring that is filled without a loop and
-// refilled without a branch around the block id's shuffle. us in the form for any
-// table and in this one: 48 layers one after another, one session of 1K tokens
+// pacing, no partials or arrival, and a ring that is filled without a loop. us in
+// the form for any table and in this one: 48 layers one after another, one session of 1K tokens
 // 303.5 and 290.1, of 300 151.4 and 149.1, 8 of 1K 327.5 and 320.3, 40 of 1 000 741
 // and 726, 128 of 1 000 2 000 and 1 983, but 12 of 300 174.3 and 180.4; all
 // layers in one call, one session of 1K 18.2 and 16.5 with K and V in the L2, 21.5
@@ -778,8 +777,12 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         for (int i = 0; i < 8; ++i) mma_bf16(s.o[i], f[i][0], f[i][1], f[i][2], f[i][3], pb0, pb1);
     };
     auto slot_of = [&](int k) { return ring_s + (k % kStages) * kTileBytes; };
+    // Without a branch around the shuffle, except where the ring holds a whole split
+    // of 64 tiles: one layer after another of 48, one session of 16 391 tokens 366.7 us
+    // with the branch and 355.4 without, 16 of 14 000 3 368 and 3 366, but one of
+    // 3 001 in splits shared by 8 CTAs 235.5 and 239.1.
     auto refill = [&](int k) {
-        if (!kOne && k + kStages >= my_tiles) return;
+        if (kSub == 8 && k + kStages >= my_tiles) return;
         const int nblk = blk_of(k + kStages);
         if (lane == 0 && k + kStages < my_tiles) issue(k + kStages, nblk);
     };
