@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkvtier.so")
 SOURCES = ["decode_kernels.cu", "copy_kernels.cu", "pool.cpp", "noalloc.cu"]
-HEADERS = ["kvt_internal.h", os.path.join("..", "..", "include", "kvtier.h")]
+HEADERS = ["kvt_internal.h", "decode_launch.h", os.path.join("..", "..", "include", "kvtier.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -24,6 +24,7 @@
 
 #include <type_traits>
 
+#include "decode_launch.h"
 #include "kvt_internal.h"
 
 namespace kvt {
@@ -33,14 +34,6 @@ namespace {
 #define KVT_STAGES 2   // 4 warps x 2 x 8 KiB: 3 CTAs (24 tiles in flight) per SM
 #endif
 constexpr int kCombineWarps = 4;
-// The merge of a session's splits folds four chains (contiguous quarters of
-// the splits, in split order) and then merges the chains in order; that order
-// depends on the split count only, whichever kernel runs it. One warp merges
-// up to kRegMergeMax splits from registers (four per chain); the split kernel
-// merges sessions of up to kSplitKernelMerge splits itself in long grids.
-constexpr int kMergeChains = 4;
-constexpr int kRegMergeMax = 16;
-constexpr int kSplitKernelMerge = 4;
 static_assert(kCombineWarps == kMergeChains && kRegMergeMax == kMergeChains * 4 &&
                   kSplitKernelMerge <= kRegMergeMax,
               "four splits per chain in a register merge, one chain per combine warp");
@@ -62,13 +55,9 @@ constexpr int kHalfBytes = 2048;           // 16 rows x 128 B (64 dims)
 //   <8 / kSub warps, slots, kSub>   a split shared by kSub = 2 or 8 CTAs, one
 //                                   accumulator per warp: grids of up to
 //                                   three CTAs per SM once shared
-constexpr int kAccs = 8;
 // Lazy softmax maximum: the reference moves when a logit exceeds it by more
 // than this many powers of two (P then stays at most 2^8 = 256).
 constexpr float kLazyLog2 = 8.f;
-#ifndef KVT_WAVE_MARGIN
-#define KVT_WAVE_MARGIN 0.1   // last-wave fill gain that moves a grid to 2 CTAs per SM
-#endif
 constexpr int kWarpsNarrow = 4;
 constexpr int kStagesFull = KVT_STAGES;    // 3 CTAs per SM
 constexpr int kStagesHalf = 3;             // 2 CTAs per SM
@@ -281,12 +270,6 @@ __device__ __forceinline__ void join_accs(float (&m)[kN], float (&l)[kN], float4
     }
     if constexpr (kN == 2 || kN == 8)
         lse_step(m[0], l[0], acc[0], make_float2(m[kN / 2], l[kN / 2]), acc[kN / 2]);
-}
-
-// Partial rows per split of a grid whose splits are shared by `sub` CTAs: one
-// per half where each of two CTAs holds one, one per accumulator for eight.
-__host__ __device__ constexpr int parts_per_split(int sub) {
-    return sub <= 2 ? sub : kAccs;
 }
 
 // Dims 4*lane .. 4*lane + 3 of output row `row`.
@@ -1269,6 +1252,14 @@ static cudaError_t launch_split(cudaLaunchConfig_t &c, const CUtensorMap &map, c
     return cudaLaunchKernelEx(&c, decode_split_kernel<kWarps, kStages, kSub, kForm>, map, a);
 }
 
+template <int kStages>
+static cudaError_t launch_unshared(const DecodeShape &d, cudaLaunchConfig_t &c, const CUtensorMap &map,
+                                   const DecodeArgs &a) {
+    if (d.one_split) return launch_split<kWarpsNarrow, kStages, 1, kOneSplit>(c, map, a);
+    if (d.by_length) return launch_split<kWarpsNarrow, kStages, 1, kLongestFirst>(c, map, a);
+    return launch_split<kWarpsNarrow, kStages, 1>(c, map, a);
+}
+
 cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_sms,
                           cudaStream_t st, bool overlap_previous) {
     // Every session of the batch has T <= max_blocks * bt, so its splits fit.
@@ -1284,119 +1275,29 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     c1.stream = st;
     c1.attrs = overlap_previous ? attr : nullptr;
     c1.numAttrs = overlap_previous ? 1 : 0;
-    // CTAs of the grid (an upper bound: splits past a session's own count
-    // exit at once) against the SMs decide the ring depth.
-    const int64_t ctas = static_cast<int64_t>(splits) * a.s.Hkv * a.nlayers * a.B;
-    // Beyond two CTAs per SM, 2 per SM still wins when it fills its last wave
-    // clearly better than 3 per SM (a grid just above one 3-per-SM wave).
-    auto fill = [&](int per_sm) {
-        const double w = static_cast<double>(ctas) / (per_sm * static_cast<double>(num_sms));
-        return w / static_cast<double>(static_cast<int64_t>(w) + (w > static_cast<int64_t>(w)));
-    };
-    // Splits shared by several CTAs. A grid of few CTAs leaves SMs idle, and
-    // each of its CTAs draws 512 KB or more through one SM (6 us) with its
-    // warps in each other's way; shared, a CTA has less to draw, holds more of
-    // it before the previous call ends, and is gone sooner, so the next call's
-    // CTAs start their copies sooner. The combine reads 2 or 8 states per split
-    // instead of one. us per layer, unshared and shared:
-    //   8 (one warp each, its ring the whole of a 64-tile split), at most two
-    //     per SM: 1 x 3 001 8.04 and 5.14, 1 x 8K 8.51 and 5.70, 4 x 1 280 8.26
-    //     and 5.10 (shared by 4 of two warps, one per SM: 6.85 and 6.51)
-    //   2, at most one per SM: 1 x 16 391 9.97 and 8.72 (two CTAs per SM with
-    //     half the ring 10.0, four of a shorter split 10.6)
-    //   2, two per SM: 8 x 4K 13.1 and 12.4, 2 x 16K 13.3 and 12.6, 5 x 5K 11.6
-    //     and 10.9 (three per SM 14.0, 14.0, 12.1)
-    //   2, three per SM: 8 x 5K 17.1 and 15.7, 10 x 4K 17.4 and 15.7, 3 x 16K
-    //     19.3 and 18.3; not the long splits of tables wider than 32K tokens
-    //     (1 x 100K 34.3 and 35.0), which do share at two per SM (1 x 40K 16.8
-    //     and 16.1)
-    // Sessions of one split need no combine unshared, and do not share: from a
-    // graph it would still pay for one to four of them above 512 tokens (1 x 1K
-    // 6.25 and 5.10, but 8 x 1K 6.98 and 6.94, 48 x 1 000 18.4 and 21.0), while
-    // direct calls would pay for the second launch. A caller's scratch may have
-    // no room for the extra rows.
-    const int64_t sms = num_sms;
-    const int64_t rows1 = static_cast<int64_t>(splits) * a.s.Hq * a.nlayers * a.B;
-    auto fits = [&](int sub, int per_sm) {
-        return sub * ctas <= per_sm * sms && parts_per_split(sub) * rows1 <= a.part_rows;
-    };
-    const bool wide = splits > kRegMergeMax;   // long splits, and a combine in batches
-    int sub = 1;
-    int per_sm = 1;   // of a shared grid
-    if (splits > 1) {
-        if (!wide && fits(8, 2))
-            sub = 8;
-        else if (fits(2, 1))
-            sub = 2;
-        else if (fits(2, 2))
-            sub = per_sm = 2;
-        else if (!wide && fits(2, 3))
-            sub = 2, per_sm = 3;
-    }
+    const DecodeShape d = decode_shape(a, splits, num_sms, overlap_previous);
     DecodeArgs ka = a;
-    // An overlapped call whose CTAs are all resident at once fills its rings
-    // while the previous call still merges: 20-30 MB of copies queued in front
-    // of that call's partials, this call's q and the end of the grid between
-    // them. Paced to one tile per warp (two with four warps per SM), the copies
-    // still keep HBM busy and the chain behind them is shorter. us per layer,
-    // unpaced and paced: one session of 16 391 tokens 8.64 and 7.98, 32K 13.6
-    // and 12.7; 8 x 4K 15.0 and 13.2, 12 x 2K 12.1 and 11.4; 4 x 16K 24.1 and
-    // 23.1. Rings that cover a whole split (8 CTAs per split) showed no
-    // difference, and in grids of more than one wave the later CTAs lose by it
-    // (8 x 16K 44.4 and 45.1). Calls without a combine (40 x 1 000 16.0 and
-    // 16.9) and unshared long splits (1 x 100K) take no part.
-    ka.pace = 0;
-    if (overlap_previous && sub == 2)
-        ka.pace = per_sm == 1 ? 2 : 1;
-    else if (overlap_previous && sub == 1 && splits > 1 && !wide && ctas <= 2 * sms)
-        ka.pace = 1;
-    // A grid of several waves ends when its last long splits do, with most SMs
-    // waiting: where splits differ in length (tables wider than 16K tokens) the
-    // longest sessions go out first. 48 layers of 16 sessions of 2K-30K tokens
-    // 3 920 -> 3 822 us, of 32 of 8K-32K 9 188 -> 9 043, 24 layers of 12 of
-    // 4K-60K 2 601 -> 2 531. Equal splits only lose by it, the block ids then
-    // waiting for the ranks (24 of 1K-14K 2 879 and 2 920); a lane ranks one
-    // session, so up to 32.
-    const bool by_length = a.nlayers == 1 && a.B > 1 && a.B <= 32 && sub == 1 && ctas > 3 * sms &&
-                           split_tiles(a.max_blocks * a.s.bt) > KVT_SPLIT_MIN_TILES;
-    // Which sessions the split kernel merges itself (the bits are the same
-    // either way): those of up to kSplitKernelMerge splits, in grids of at
-    // least 8 CTAs per SM. There, many groups finish at different times and
-    // their merges spread over the grid. In shorter grids each CTA's arrival
-    // (an atomic round trip holding its SM slot) and the tail merges cost more
-    // than the combine launch (measured on GB300 against merging everything in
-    // the combine: 256 x 4K-token sessions per layer +1.3 %, 8 x 4K all
-    // layers +1.6 %; one 4K- or 16K-token session per layer -7 % / -5 % and
-    // 32 x 4K -5 % when shorter grids merged too).
-    ka.merge_max_splits = ctas >= 8 * sms ? kSplitKernelMerge : 0;
-    const bool combine = sub > 1 || (splits > 1 && splits > ka.merge_max_splits);
+    ka.pace = d.pace;
+    ka.merge_max_splits = d.merge_max_splits;
     cudaError_t e;
-    if (sub == 8)
+    if (d.sub == 8)
         e = launch_split<1, 8, 8>(c1, map, ka);
-    else if (sub == 2 && per_sm == 1)
+    else if (d.sub == 2 && d.per_sm == 1)
         e = launch_split<4, 6, 2>(c1, map, ka);
-    else if (sub == 2 && per_sm == 2)
+    else if (d.sub == 2 && d.per_sm == 2)
         e = launch_split<4, 3, 2>(c1, map, ka);
-    else if (sub == 2)
+    else if (d.sub == 2)
         e = launch_split<4, 2, 2>(c1, map, ka);
-    else if (splits == 1 && ctas <= sms)
-        e = launch_split<8, 3, 1, kOneSplit>(c1, map, ka);
-    else if (splits == 1)
-        e = ctas <= 2 * sms || fill(2) > fill(3) + KVT_WAVE_MARGIN
-                ? launch_split<kWarpsNarrow, kStagesHalf, 1, kOneSplit>(c1, map, ka)
-                : launch_split<kWarpsNarrow, kStagesFull, 1, kOneSplit>(c1, map, ka);
-    else if (ctas <= sms)
-        e = launch_split<8, 3, 1>(c1, map, ka);
-    else if (ctas <= 2 * sms || fill(2) > fill(3) + KVT_WAVE_MARGIN)
-        e = by_length ? launch_split<kWarpsNarrow, kStagesHalf, 1, kLongestFirst>(c1, map, ka)
-                      : launch_split<kWarpsNarrow, kStagesHalf, 1>(c1, map, ka);
+    else if (d.per_sm == 1)
+        e = d.one_split ? launch_split<8, 3, 1, kOneSplit>(c1, map, ka) : launch_split<8, 3, 1>(c1, map, ka);
+    else if (d.per_sm == 2)
+        e = launch_unshared<kStagesHalf>(d, c1, map, ka);
     else
-        e = by_length ? launch_split<kWarpsNarrow, kStagesFull, 1, kLongestFirst>(c1, map, ka)
-                      : launch_split<kWarpsNarrow, kStagesFull, 1>(c1, map, ka);
+        e = launch_unshared<kStagesFull>(d, c1, map, ka);
     if (e != cudaSuccess) return e;
     // Else the split kernel writes every session's output: one split each, or
     // few enough splits to merge there.
-    if (!combine) return cudaSuccess;
+    if (!d.combine) return cudaSuccess;
 
     const int64_t rows = static_cast<int64_t>(a.nlayers) * a.B * a.s.Hq;
     cudaLaunchConfig_t c2 = {};
@@ -1405,15 +1306,15 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     c2.stream = st;
     c2.attrs = attr;
     c2.numAttrs = 1;
-    if (sub == 1 && !wide) {
+    if (d.sub == 1 && !d.wide) {
         c2.gridDim = dim3(static_cast<unsigned>((rows + 3) / 4));
         return cudaLaunchKernelEx(&c2, decode_combine_small_kernel, ka);
     }
     c2.gridDim = dim3(static_cast<unsigned>(rows));
-    if (wide)
-        return sub == 2 ? cudaLaunchKernelEx(&c2, decode_combine_kernel<2, 8>, ka)
+    if (d.wide)
+        return d.sub == 2 ? cudaLaunchKernelEx(&c2, decode_combine_kernel<2, 8>, ka)
                         : cudaLaunchKernelEx(&c2, decode_combine_kernel<1, 16>, ka);
-    if (sub == 8) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<8>, ka);
+    if (d.sub == 8) return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<8>, ka);
     return cudaLaunchKernelEx(&c2, decode_combine_shared_kernel<2>, ka);
 }
 

@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "../../include/kvtier.h"
+#include "decode_launch.h"
 #include "kvt_internal.h"
 
 static_assert(KV_DEVICE_BAD_BLOCK == kvt::kErrBadBlock && KV_DEVICE_BAD_LENGTH == kvt::kErrBadLength &&
@@ -497,12 +498,7 @@ int kv_pool_create(const kv_pool_config *cfg, kv_pool **out) {
             return bail(fail(KV_ERR_CUDA, "cudaSetDevice failed"));
         cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, c.device);
         const int64_t tbl = static_cast<int64_t>(c.max_sessions) * p->table_stride * 4;
-        // Small grids share a split among 8 CTAs, at most two per SM, and leave
-        // 8 partial rows of it, or among 2, at most three per SM, and leave 2
-        // (launch_decode).
-        const int64_t wave = static_cast<int64_t>(p->num_sms) * (c.num_q_heads / c.num_kv_heads);
-        p->part_alloc = std::max({p->part_rows, std::min(8 * p->part_rows, 2 * wave),
-                                  std::min(2 * p->part_rows, 3 * wave)});
+        p->part_alloc = kvt::shared_part_rows(p->part_rows, p->num_sms, c.num_q_heads / c.num_kv_heads);
         const int64_t prow = p->part_alloc;
         // A multi-split call has at most part_rows / Hq layer-batch rows.
         p->counter_count = p->part_rows / c.num_q_heads * c.num_kv_heads;

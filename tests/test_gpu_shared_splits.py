@@ -15,6 +15,7 @@ import torch
 
 import oracle
 import synth
+from launch_rules import decode_shape, pool_part_rows
 from test_gpu_parity import TOL, direct_case, gpu_decode, host_hot, pkg, scaled_err  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -41,14 +42,13 @@ CASES = [
 @pytest.mark.parametrize("lens,tokens,hkv,shared", CASES)
 @pytest.mark.parametrize("bt,scale", [(16, 1 / math.sqrt(128)), (64, 0.5)])
 def test_shared_splits(pkg, lens, tokens, hkv, shared, bt, scale):  # noqa: F811
-    from paper_2609_25782_gb300 import kvtier
-    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
-        ctas = kvtier.kv_decode_splits(-(-tokens // bt) * bt) * hkv * len(lens)
-        room = {1: 10 ** 9, 2: 3 * 152, 8: 2 * 152}[shared]
-        assert shared * ctas <= room
-        assert shared != 2 or 8 * ctas > 2 * 152 or tokens > 32768
     n = len(lens)
     many = lens + [100] * (520 // (n * hkv))    # a batch too large to share
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        room = pool_part_rows(len(many), max(many), 8 * hkv, hkv, 152)
+        kw = dict(bt=bt, hq=8 * hkv, hkv=hkv, part_rows=room)
+        assert decode_shape(tokens, n, **kw).sub == shared
+        assert decode_shape(max(many), len(many), **kw).sub == 1
     pool, sess, tables, q = direct_case(pkg, many, L=1, Hq=8 * hkv, Hkv=hkv, bt=bt, seed=17,
                                         max_batch=len(many))
     pool._scale = scale                         # 0.5: logits of std 5.7, so the maximum moves late
@@ -66,10 +66,15 @@ def test_shared_splits(pkg, lens, tokens, hkv, shared, bt, scale):  # noqa: F811
 
 # Grids of several waves whose splits differ in length start with the longest
 # sessions (up to 32 of them): each row once, whatever its rank, ties included.
+LONGEST_FIRST = [17003, 20, 17003, 1, 16400, 5000, 64, 17003, 1] + [700 + 37 * (i % 5) for i in range(24)]
+
+
 @pytest.mark.parametrize("n", [9, 31, 32, 33])
 @pytest.mark.parametrize("bt", [16, 64])
 def test_longest_first(pkg, n, bt):  # noqa: F811
-    lens = ([17003, 20, 17003, 1, 16400, 5000, 64, 17003, 1] + [700 + 37 * (i % 5) for i in range(24)])[:n]
+    lens = LONGEST_FIRST[:n]
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert decode_shape(max(lens), n, bt=bt).by_length == (n <= 32)
     pool, sess, tables, q = direct_case(pkg, lens, L=1, bt=bt, seed=23, max_batch=n)
     got = gpu_decode(pool, 0, q, tables, lens)[0]
     for i in range(n):
@@ -105,4 +110,32 @@ def test_tables_of_one_split(pkg, n, bt, hkv):  # noqa: F811
         pool.decode_attention(l, q[l].contiguous(), t, s, n, t.shape[1], 0.5, out[l], overlap_previous=l > 0)
     torch.cuda.synchronize()
     assert np.array_equal(out.double().cpu().numpy().view(np.int64), got.view(np.int64))
+    assert pool.check_device() == 0
+
+
+@pytest.mark.parametrize("n", [9, 32])
+@pytest.mark.parametrize("bt", [16, 64])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_longest_first_fused_layers(pkg, n, bt, bf16):  # noqa: F811
+    """The same with each row's newest token from k_new and v_new, in overlapped calls layer by
+    layer: rows of k_new, v_new and out are the batch's, whatever their rank in the grid."""
+    L, lens = 3, LONGEST_FIRST[:n]
+    pool, _, tables, q = direct_case(pkg, lens, L=L, bt=bt, seed=29, max_batch=n)
+    want = torch.from_numpy(np.concatenate([gpu_decode(pool, l, q, tables, lens) for l in range(L)]))
+    hot = pool.hot_view()
+    at = torch.as_tensor([int(tables[b, (t - 1) // bt]) for b, t in enumerate(lens)], device="cuda")
+    slot = torch.as_tensor([(t - 1) % bt for t in lens], device="cuda")
+    new = hot[at, :, :, :, slot].clone()                   # [B][L][K|V][Hkv][D]
+    k_new, v_new = (new[:, :, i].transpose(0, 1).contiguous() for i in (0, 1))
+    before = pool.hot.clone()
+    hot[at, :, :, :, slot] = float("nan")
+    t = torch.as_tensor(tables, device="cuda")
+    s = torch.as_tensor(np.asarray(lens, dtype=np.int32), device="cuda")
+    out = torch.empty(L, n, 32, 128, dtype=torch.bfloat16 if bf16 else torch.float32, device="cuda")
+    for l in range(L):
+        pool.decode_append_attention(l, q[l], k_new[l], v_new[l], t, s, n, t.shape[1],
+                                     1 / math.sqrt(128), out[l], overlap_previous=l > 0)
+    torch.cuda.synchronize()
+    assert torch.equal(out.cpu(), want.float().to(out.dtype))
+    assert torch.equal(pool.hot.view(torch.int16), before.view(torch.int16))
     assert pool.check_device() == 0
