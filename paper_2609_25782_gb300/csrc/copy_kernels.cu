@@ -22,9 +22,10 @@ namespace {
 
 // Migration copy shape: one warp per 8-token chunk of a run (2 KiB on both
 // sides), moved by one round of 32-byte loads, two per lane, and stores. Bound
-// by HBM. The warps are not reused: a grid-stride loop over 32 CTAs per SM moved
-// three sessions of 20K-30K tokens in 2.26 ms, one warp per chunk in 2.19 ms
-// (its 16-byte predecessor in 2.31 ms, 1.00 of the copy bandwidth). Four loads
+// by HBM. The warps are not reused, unless decode may run beside the move
+// (migration_ctas): a grid-stride loop over 32 CTAs per SM moved three sessions of
+// 20K-30K tokens in 2.26 ms, one warp per chunk in 2.19 ms (16-byte loads in
+// that loop 2.31 ms). Four loads
 // per lane over 16 tokens need 48 registers, so five CTAs an SM instead of
 // six, and a move of 29 MB ends with a second wave of a few CTAs: two resumes of
 // 892 tokens, 16 layers, 28.4 us, now 26.1 (27.6 with 16-byte loads); of 1 000
@@ -142,8 +143,6 @@ __device__ __forceinline__ void migrate_runs(const MigArgs &a, BlockOf block_of)
     }
 }
 
-// K3'/K4': block-granular moves for the residency mode: one warp per
-// (job, layer, K|V, kv-head) run; a job moves tokens [t0, t1) of one block.
 template <bool kPack>
 __global__ void __launch_bounds__(kCopyThreads) migrate_kernel(const MigArgs a) {
     migrate_runs<kPack>(a, [&](int j) { return a.table[j]; });
@@ -159,6 +158,8 @@ __global__ void __launch_bounds__(kCopyThreads) resume_inline_kernel(const __gri
     migrate_runs<false>(r.m, [&](int j) { return j < r.n ? r.blocks[j] : -1; });
 }
 
+// K3'/K4': block-granular moves for the residency mode: one warp per chunk of a
+// (job, layer, K|V, kv-head) run; a job moves tokens [t0, t1) of one block.
 template <bool kPack>
 __global__ void __launch_bounds__(kCopyThreads) block_jobs_kernel(const __grid_constant__ BlockJobs a) {
     const Shape sh = a.s;

@@ -48,10 +48,10 @@ constexpr int kHalfBytes = 2048;           // 16 rows x 128 B (64 dims)
 //                                   and w + 4 and alternates between them, so
 //                                   consecutive tiles of a warp are independent
 //   <4 warps, 3 slots, 1>           2 CTAs per SM
-//   <8 warps, 3 slots, 1>           1 CTA per SM: one accumulator per warp,
+//   these two, kLongestFirst        their CTAs take the longest sessions first
+//   these two, kOneSplit            tables of one split (kernel forms, below)
+//   <8 warps, 3 slots, 1, kOneSplit>   1 CTA per SM: one accumulator per warp,
 //                                   twice the warps per SM
-//   the first two, kLongestFirst    their CTAs take the longest sessions first
-//   these three, kOneSplit          tables of one split (kernel forms, below)
 //   <8 / kSub warps, slots, kSub>   a split shared by kSub = 2 or 8 CTAs, one
 //                                   accumulator per warp: grids of up to
 //                                   three CTAs per SM once shared
@@ -1233,7 +1233,6 @@ cudaError_t prepare_kernels() {
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1>();
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1, kLongestFirst>();
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1, kLongestFirst>();
-    if (e == cudaSuccess) e = prepare_split<8, 3, 1>();
     if (e == cudaSuccess) e = prepare_split<8, 3, 1, kOneSplit>();
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesHalf, 1, kOneSplit>();
     if (e == cudaSuccess) e = prepare_split<kWarpsNarrow, kStagesFull, 1, kOneSplit>();
@@ -1289,7 +1288,7 @@ cudaError_t launch_decode(const CUtensorMap &map, const DecodeArgs &a, int num_s
     else if (d.sub == 2)
         e = launch_split<4, 2, 2>(c1, map, ka);
     else if (d.per_sm == 1)
-        e = d.one_split ? launch_split<8, 3, 1, kOneSplit>(c1, map, ka) : launch_split<8, 3, 1>(c1, map, ka);
+        e = launch_split<8, 3, 1, kOneSplit>(c1, map, ka);
     else if (d.per_sm == 2)
         e = launch_unshared<kStagesHalf>(d, c1, map, ka);
     else

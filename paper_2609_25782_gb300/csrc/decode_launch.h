@@ -83,7 +83,7 @@ inline DecodeShape decode_shape(const DecodeArgs &a, int splits, int num_sms, bo
     //     and 16.1)
     // Sessions of one split need no combine unshared, and do not share: from a
     // graph it would still pay for one to four of them above 512 tokens (1 x 1K
-    // 6.25 and 5.10, but 8 x 1K 6.98 and 6.94, 48 x 1 000 18.4 and 21.0), while
+    // 6.04 and 5.10, but 8 x 1K 6.67 and 6.94, 48 x 1 000 18.4 and 21.0), while
     // direct calls would pay for the second launch. A caller's scratch may have
     // no room for the extra rows.
     const int64_t sms = num_sms;
@@ -102,7 +102,7 @@ inline DecodeShape decode_shape(const DecodeArgs &a, int splits, int num_sms, bo
     } else if (splits > 1 && (fits(2, 1) || fits(2, 2) || (!wide && fits(2, 3)))) {
         d.sub = 2;
         d.per_sm = fits(2, 1) ? 1 : fits(2, 2) ? 2 : 3;
-    } else if (ctas <= sms) {
+    } else if (d.one_split && ctas <= sms) {
         d.per_sm = 1;
     } else {
         d.per_sm = ctas <= 2 * sms || fill(2) > fill(3) + KVT_WAVE_MARGIN ? 2 : 3;

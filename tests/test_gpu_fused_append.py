@@ -15,6 +15,7 @@ import torch
 
 import oracle
 import synth
+from launch_rules import decode_shape
 
 pytestmark = pytest.mark.gpu
 
@@ -163,13 +164,23 @@ def test_fused_steps_cross_blocks_and_splits(pkg):
 
 
 def test_fused_steps_one_cta_per_sm(pkg):
-    """A batch small enough for one CTA per SM (3 splits x 4 kv-heads x 3
-    sessions = 36 CTAs) runs the 8-warp kernel, one accumulator per warp,
-    while larger grids run 4 warps with two accumulators each. Over twenty
-    steps the token that arrives with the call lands in different warps and
-    accumulators; the fused run stays bit-identical to append-then-decode
-    and agrees with the oracle."""
-    lens = [70, 1100, 2030]
+    """A batch of few CTAs (3 splits x 4 kv-heads x 3 sessions = 36) shares
+    each split among 8, one accumulator each, while larger grids run 4 warps
+    with two accumulators each. Over twenty steps the token that arrives with
+    the call lands in different CTAs and accumulators; the fused run stays
+    bit-identical to append-then-decode and agrees with the oracle."""
+    small_fused_run(pkg, [70, 1100, 2030], 8)
+
+
+def test_fused_steps_tables_of_one_split(pkg):
+    """The same in tables of one split, whose CTAs have 8 warps, one accumulator each."""
+    small_fused_run(pkg, [70, 15, 1000], 1)
+
+
+def small_fused_run(pkg, lens, shared):
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        d = decode_shape(max(lens) + 21, len(lens))
+        assert d.sub == shared and d.one_split == (shared == 1)
     pf, sids, T, of, q = run(pkg, True, lens, 20, L=2, mode="layer")
     pu, _, _, ou, _ = run(pkg, False, lens, 20, L=2, mode="layer")
     for a, b in zip(of, ou):

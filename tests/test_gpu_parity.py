@@ -13,6 +13,7 @@ import torch
 
 import oracle
 import synth
+from launch_rules import decode_shape
 
 pytestmark = pytest.mark.gpu
 
@@ -140,21 +141,25 @@ def test_decode_independent_of_batch_and_placement(pkg):
 
 
 def test_ring_depths_bit_identical(pkg):
-    """The split kernel's launch variant follows the size of the grid: one
-    CTA per SM with 8 warps (one of a split's eight accumulators each), or 2
-    or 3 CTAs per SM with 4 warps (two accumulators each) and 3- or 2-deep
-    tile rings. The variants change where the accumulators run and how far
-    ahead tiles are fetched, never which tiles an accumulator takes or the
-    merge order, so all must give the same bits."""
+    """The split kernel's launch variant follows the size of the grid: splits
+    shared by two CTAs of 4 warps (one of a split's eight accumulators each)
+    at one, two or three CTAs per SM with 6-, 3- or 2-deep tile rings, or
+    CTAs of 4 warps with two accumulators each. The variants change where the
+    accumulators run and how far ahead tiles are fetched, never which tiles
+    an accumulator takes or the merge order, so all must give the same bits."""
     lens = [5000, 3001, 777]
     L = 16
     pool, sess, tables, q = direct_case(pkg, lens, L=L, seed=4, max_batch=L * len(lens))
     mid = np.pad(tables, ((0, 0), (0, 600 - tables.shape[1])), constant_values=-1)
     wide = np.pad(tables, ((0, 0), (0, 2048 - tables.shape[1])), constant_values=-1)
-    # per layer, 313-block tables: 5 splits x 4 kv-heads x 3 rows = 60 CTAs (8 warps);
-    # per layer, 600-block tables: 10 x 4 x 3 = 120 CTAs (8 warps);
-    # per layer, tables 2048 blocks wide: 16 x 4 x 3 = 192 CTAs (4 warps, 3-deep);
-    # all 16 layers in one call: 5 x 4 x 48 = 960 CTAs (4 warps, 2-deep)
+    # unshared, per layer, 313-block tables are 5 splits x 4 kv-heads x 3 rows = 60 CTAs,
+    # 600-block tables 10 x 4 x 3 = 120, tables 2 048 blocks wide 16 x 4 x 3 = 192, all
+    # 16 layers in one call 5 x 4 x 48 = 960
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        for tokens, layers, want in ((5008, 1, (2, 1)), (9600, 1, (2, 2)), (32768, 1, (2, 3)),
+                                     (5008, L, (1, 3))):
+            d = decode_shape(tokens, 3, layers=layers)
+            assert (d.sub, d.per_sm) == want
     narrow = np.concatenate([gpu_decode(pool, l, q, tables, lens) for l in range(L)])
     middle = np.concatenate([gpu_decode(pool, l, q, mid, lens) for l in range(L)])
     padded = np.concatenate([gpu_decode(pool, l, q, wide, lens) for l in range(L)])
