@@ -510,6 +510,7 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
     static_assert(kWarps * kStages * 8 <= 256, "mbarriers must fit their 256-byte area");
     constexpr bool kOne = kForm == kOneSplit;
     static_assert(!kOne || kSub == 1, "one split: unshared");
+    constexpr bool kPaced = kForm == kAny && (kSub == 2 || (kSub == 1 && kStages == kStagesHalf));
     static_assert(kA * kStep == kAccs, "accumulators divide among the warps");
     static_assert(kA == 1 || (kA == 2 && kSub == 1), "two accumulators only in an unshared split");
     extern __shared__ uint8_t smem_raw[];
@@ -631,9 +632,10 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
 #pragma unroll 1
         for (int k = from; k < to; ++k) mbar_wait(bar0 + 8 * (k % kStages), (k / kStages) & 1);
     };
-    // a.pace > 0 (launch_decode): at most that many of the warp's tiles in
-    // flight while the previous kernel may still be running. A warp whose wait
-    // runs out here issues no more, and has no tiles to consume.
+    // The ring's first tiles. a.pace > 0 (decode_shape; the other forms do not carry
+    // it): at most that many of the warp's tiles in flight while the previous
+    // kernel may still be running. A warp whose wait runs out here issues no more,
+    // and has no tiles to consume.
     if constexpr (kOne) {
 #pragma unroll
         for (int k = 0; k < kStages; ++k) {
@@ -642,16 +644,16 @@ __global__ void __launch_bounds__(kWarps * 32, kWarps != kWarpsNarrow ? 1 : kSta
         }
     } else {
 #pragma unroll 1
-    for (int k = 0; k < kStages && k < my_tiles; ++k) {
-        const int blk = blk_of(k);
-        if (a.pace > 0 && k >= a.pace &&
-            !__all_sync(0xffffffffu, mbar_wait(bar0 + 8 * (k - a.pace), 0))) {
-            give_up(k - a.pace, k);
-            my_tiles = 0;
-            break;
+        for (int k = 0; k < kStages && k < my_tiles; ++k) {
+            const int blk = blk_of(k);
+            if (kPaced && a.pace > 0 && k >= a.pace &&
+                !__all_sync(0xffffffffu, mbar_wait(bar0 + 8 * (k - a.pace), 0))) {
+                give_up(k - a.pace, k);
+                my_tiles = 0;
+                break;
+            }
+            if (lane == 0) issue(k, blk);
         }
-        if (lane == 0) issue(k, blk);
-    }
     }
 
     uint32_t koff[4], voff[4];

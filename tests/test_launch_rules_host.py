@@ -73,6 +73,8 @@ def test_decode_shape(case, want):
         assert (d.sub, d.per_sm, d.merge_max, d.one_split, d.by_length, d.combine) == \
             (sub, per_sm, merge, one, first, combine)
         assert d.pace == (pace if overlap else 0)
+        # the kernels that carry the pacing
+        assert not d.pace or d.sub == 2 or ((d.sub, d.per_sm) == (1, 2) and not d.one_split and not d.by_length)
         assert d.wide == (splits_of(tokens) > 16)
 
 
@@ -99,6 +101,8 @@ def test_decode_shape_keeps_to_the_workspace():
         for room in (rows, 2 * rows - 1, 2 * rows, 8 * rows - 1, 8 * rows):
             d = decode_shape(tokens, batch, part_rows=room, **c)
             assert d.sub * rows <= room          # 2 or 8 rows of a shared split
+            assert not d.pace or d.sub == 2 or ((d.sub, d.per_sm) == (1, 2) and not d.one_split
+                                                and not d.by_length)
             shared.add((room // rows, d.sub))
     assert shared == {(1, 1), (2, 1), (2, 2), (7, 1), (7, 2), (8, 1), (8, 2), (8, 8)}
 
